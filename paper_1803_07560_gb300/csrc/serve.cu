@@ -370,9 +370,11 @@ void finish_pass(bfi_server *s, Pass &p, const double *stage) {
     const bfi_status ms = bfi_merge_host(r.lat.nx, static_cast<int64_t>(r.leaf_sid.size()), r.leaf_slots.data(),
                                          r.totals.data());
     rl.unlock();
+    {  // counted before the request ends: a caller whose wait has returned sees it
+        std::lock_guard<std::mutex> lock(s->m);
+        s->st.completed++;
+    }
     end_request(r, ms == BFI_OK ? 2 : 4, ms, ms == BFI_OK ? nullptr : "merge failed");
-    std::lock_guard<std::mutex> lock(s->m);
-    s->st.completed++;
 }
 
 // A pass that failed after admission: its job fails with 'status', its
