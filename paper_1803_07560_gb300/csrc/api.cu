@@ -136,12 +136,15 @@ ChunkLayout plan_chunk_layout(const uint64_t *samples, int64_t nsub) {
 float plan_negligible_window(bfi_precision precision, uint64_t n_max) { return negligible_window(precision, n_max); }
 }  // namespace bfi
 
+constexpr size_t kPlanCounters = 5;
+
 struct bfi_plan {
     int device = 0;
     bfi::LatticeParams lat{};
     bfi_precision precision = BFI_FP64;
     const bfi::ShapeKernels *shape = nullptr;
     int64_t nsub = 0, nchunks = 0, chunk_samples = 0, total = 0;
+    int64_t windows = 0;  // of the merge
     bfi::ChunkLayout layout;
     int grid = 1;
     int sms = 1, per_sm_max = 1, per_sm = 1;
@@ -151,7 +154,7 @@ struct bfi_plan {
     uint64_t *d_samples = nullptr;
     double *d_partials = nullptr;
     float *d_hint = nullptr;
-    unsigned long long *d_stats = nullptr;
+    unsigned long long *d_stats = nullptr;  // evaluated, fully screened, stage 1, next chunk, merge arrivals
     double *d_fbuf = nullptr;
     float skip_window = 0.f;
     size_t scratch_bytes = 0;
@@ -231,9 +234,14 @@ bfi_status bfi_plan_create(bfi_plan **out, const bfi_lattice *lattice, int64_t n
     for (int64_t s = 0; s < nsub; ++s) n_max = std::max<uint64_t>(n_max, samples[s]);
     p->skip_window = negligible_window(precision, n_max);
     std::vector<int64_t> off(nsub + 1, 0);
-    for (int64_t s = 0; s < nsub; ++s)
-        off[s + 1] = off[s] + p->layout.chunks_of(s, samples[s]);
+    int64_t most = 0;
+    for (int64_t s = 0; s < nsub; ++s) {
+        const int64_t c = p->layout.chunks_of(s, samples[s]);
+        off[s + 1] = off[s] + c;
+        most = std::max(most, c);
+    }
     p->nchunks = off[nsub];
+    p->windows = bfi::merge_windows(most, p->nchunks);
 
     int sms = 0, per_sm = 0;
     cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
@@ -252,10 +260,10 @@ bfi_status bfi_plan_create(bfi_plan **out, const bfi_lattice *lattice, int64_t n
     const size_t smp_bytes = sizeof(uint64_t) * nsub;
     const size_t par_bytes = sizeof(double) * static_cast<size_t>(std::max<int64_t>(p->nchunks, 1)) * (p->K + 2);
     const size_t hint_bytes = sizeof(float) * nsub;
-    p->scratch_bytes = off_bytes + smp_bytes + par_bytes + hint_bytes + 4 * sizeof(unsigned long long) + sizeof(double) * 2 * nsub;
+    p->scratch_bytes = off_bytes + smp_bytes + par_bytes + hint_bytes + kPlanCounters * sizeof(unsigned long long) + sizeof(double) * 2 * nsub;
     if (cudaMalloc(&p->d_chunk_off, off_bytes) != cudaSuccess || cudaMalloc(&p->d_samples, smp_bytes) != cudaSuccess ||
         cudaMalloc(&p->d_partials, par_bytes) != cudaSuccess || cudaMalloc(&p->d_hint, hint_bytes) != cudaSuccess ||
-        cudaMalloc(&p->d_stats, 4 * sizeof(unsigned long long)) != cudaSuccess ||
+        cudaMalloc(&p->d_stats, kPlanCounters * sizeof(unsigned long long)) != cudaSuccess ||
         cudaMalloc(&p->d_fbuf, sizeof(double) * 2 * nsub) != cudaSuccess) {
         cudaGetLastError();
         bfi_plan_destroy(p);
@@ -318,7 +326,7 @@ bfi_status bfi_plan_execute(bfi_plan *plan, const double *lo, const double *hi, 
     if (g.err != cudaSuccess) return fail(BFI_E_CUDA, "cannot select device: %s", cudaGetErrorString(g.err));
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     if (plan->timing) BFI_CUDA(cudaEventRecord(plan->ev[0], st));
-    BFI_CUDA(cudaMemsetAsync(plan->d_stats, 0, 4 * sizeof(unsigned long long), st));
+    BFI_CUDA(cudaMemsetAsync(plan->d_stats, 0, kPlanCounters * sizeof(unsigned long long), st));
     if (plan->nchunks > 0) {
         bfi::IntegrandArgs a{lo,           hi,           sub_id,        plan->d_samples,     plan->d_chunk_off,
                              plan->d_partials, plan->d_hint, plan->d_stats, plan->nsub, plan->nchunks,
@@ -337,10 +345,10 @@ bfi_status bfi_plan_execute(bfi_plan *plan, const double *lo, const double *hi, 
         }
     }
     if (plan->timing) BFI_CUDA(cudaEventRecord(plan->ev[1], st));
-    bfi::MergeArgs m{lo, hi, plan->d_chunk_off, plan->d_partials, slots, plan->nsub, plan->R, plan->d,
-                     plan->sampler == BFI_SAMPLE_GAUSSIAN ? 1 : 0, plan->log_norm};
-    bfi::TotalsArgs t{slots, totals, plan->d_fbuf, plan->nsub, plan->R};
-    BFI_CUDA(bfi::launch_merges(m, t, st));
+    const bfi::MergeArgs m{lo, hi, plan->d_samples, plan->d_chunk_off, plan->d_partials, slots, totals, plan->d_fbuf,
+                           plan->d_stats + 4, plan->nsub, plan->windows, plan->R, plan->d, 1.0 / plan->d,
+                           plan->sampler == BFI_SAMPLE_GAUSSIAN ? 1 : 0, plan->log_norm};
+    BFI_CUDA(bfi::launch_merges(m, st));
     if (plan->timing) {
         BFI_CUDA(cudaEventRecord(plan->ev[2], st));
         plan->timed = true;
@@ -744,7 +752,7 @@ bfi_status bfi_integrate(bfi_ctx *ctx, const bfi_lattice *lattice, int64_t nsub,
 }
 
 // ---------------------------------------------------------------------------
-// Host FP64 merge: the same definitions as the device merge (merge_totals).
+// Host FP64 merge: the same definitions as the device merge (merge_slots).
 // ---------------------------------------------------------------------------
 bfi_status bfi_merge_host(int32_t nx, int64_t nsub, const double *slots, double *totals) {
     if (nx < 2 || nsub < 0 || !slots || !totals) return fail(BFI_E_INVALID, "bad arguments to bfi_merge_host");
@@ -759,8 +767,7 @@ bfi_status bfi_merge_host(int32_t nx, int64_t nsub, const double *slots, double 
         used += 1.0;
         if (q[3] > 0.0) L = std::fmax(L, q[2] - std::log(q[0]) - q[1]);
     }
-    // f_s and g_s = f_s^2 / (n_s - 1), the factor of every variance term (the
-    // same arithmetic as the device merge)
+    // f_s and g_s = f_s^2 / (n_s - 1), the factor of every variance term
     std::vector<double> f(static_cast<size_t>(nsub), 0.0), g(static_cast<size_t>(nsub), 0.0);
     double Z = 0.0, VZ = 0.0;
     for (int64_t s = 0; s < nsub; ++s) {

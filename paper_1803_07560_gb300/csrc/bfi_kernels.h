@@ -51,23 +51,30 @@ struct IntegrandArgs {
     int64_t tail_chunk_samples;    // (0: every subvolume into chunks of chunk_samples)
 };
 
+// Subvolumes of up to kMergeWhole chunks are merged by one warp; larger ones
+// in pieces of kMergePiece chunks, a warp each.  Measured on GB300 with 37
+// subvolumes of 53 chunks (7x3): 735 us a pass at 64 and at 128, 781 us at 32,
+// where the last CTA gets pieces to merge and the subvolumes to finish.
+constexpr int64_t kMergeWhole = 64, kMergePiece = 32;
+// The windows of kMergePiece chunks that the merge needs warps for.
+inline int64_t merge_windows(int64_t max_chunks_of_a_subvolume, int64_t nchunks) {
+    return max_chunks_of_a_subvolume > kMergeWhole ? (nchunks + kMergePiece - 1) / kMergePiece : 0;
+}
+
 struct MergeArgs {
     const double *lo, *hi;
-    const int64_t *chunk_off;
-    const double *partials;
-    double *slots;
+    const uint64_t *samples;       // [nsub]
+    const int64_t *chunk_off;      // [nsub + 1]
+    double *partials;              // overwritten: merged pieces, then what the totals need of each subvolume
+    double *slots, *totals;
+    double *f_buf;                 // [2 nsub] scratch: per-subvolume scale factors f_s, then f_s^2 / (n_s - 1)
+    unsigned long long *arrived;   // [1] zeroed per execution: CTAs that have merged their subvolumes
     int64_t nsub;
+    int64_t windows;               // merge_windows(...) of the job
     int32_t R, d;
-    int32_t log_norm_set;      // 1: every record's log-volume is log_norm (Gaussian sampler)
+    double inv_d;                  // 1 / d
+    int32_t log_norm_set;          // 1: every record's log-volume is log_norm (Gaussian sampler)
     double log_norm;
-};
-
-struct TotalsArgs {
-    const double *slots;
-    double *totals;
-    double *f_buf;             // [2 nsub] scratch: per-subvolume scale factors f_s, then f_s^2 / (n_s - 1)
-    int64_t nsub;
-    int32_t R;
 };
 
 struct PointsArgs {
@@ -118,7 +125,7 @@ const ShapeKernels *shapes_config_c(int *n);
 const ShapeKernels *shapes_config_d(int *n);
 const ShapeKernels *generic_shape(int nx, int nt);
 const ShapeKernels *find_shape(int nx, int nt);
-cudaError_t launch_merges(const MergeArgs &m, const TotalsArgs &t, cudaStream_t st);
+cudaError_t launch_merges(const MergeArgs &m, cudaStream_t st);
 
 // Mapped samplers (generic.cu): kind 1 = the range map of Sec. 4, kind 2 =
 // Gaussian importance sampling with device mean [d] (or null) and factor [d*d].

@@ -40,6 +40,9 @@ double ms_between(Clock::time_point a, Clock::time_point b) {
     return std::chrono::duration<double, std::milli>(b - a).count();
 }
 
+// evaluated, fully screened, stage 1, next chunk, merge arrivals
+constexpr size_t kCounters = 5;
+
 size_t round_up(size_t x) { return (x + 255) & ~size_t(255); }
 
 struct Request {
@@ -75,7 +78,7 @@ struct Pass {
     std::vector<uint64_t> samples;
     std::vector<uint32_t> sid;
     std::vector<int64_t> off;  // chunk table
-    int64_t nchunks = 0;
+    int64_t nchunks = 0, windows = 0;
     bfi::ChunkLayout chunks;
     float window = 0.f;
     Layout L{};
@@ -87,7 +90,7 @@ Layout layout_for(int64_t nsub, int64_t nchunks, int d, int K, int SL, int TL) {
     L.off = o;   o += round_up(sizeof(int64_t) * (nsub + 1));
     L.smp = o;   o += round_up(sizeof(uint64_t) * nsub);
     L.hint = o;  o += round_up(sizeof(float) * nsub);
-    L.stats = o; o += round_up(4 * sizeof(unsigned long long));  // evaluated, fully screened, stage 1, next chunk
+    L.stats = o; o += round_up(kCounters * sizeof(unsigned long long));
     L.fbuf = o;  o += round_up(sizeof(double) * 2 * nsub);
     L.part = o;  o += round_up(sizeof(double) * static_cast<size_t>(nchunks > 0 ? nchunks : 1) * (K + 2));
     L.lo = o;    o += round_up(sizeof(double) * nsub * d);
@@ -116,8 +119,14 @@ void finalize_pass(Pass &p, bfi_precision precision) {
     }
     p.chunks = bfi::plan_chunk_layout(p.samples.data(), p.nsub);
     p.off.assign(p.nsub + 1, 0);
-    for (int64_t s = 0; s < p.nsub; ++s) p.off[s + 1] = p.off[s] + p.chunks.chunks_of(s, p.samples[s]);
+    int64_t most = 0;
+    for (int64_t s = 0; s < p.nsub; ++s) {
+        const int64_t c = p.chunks.chunks_of(s, p.samples[s]);
+        p.off[s + 1] = p.off[s] + c;
+        most = std::max(most, c);
+    }
     p.nchunks = p.off[p.nsub];
+    p.windows = bfi::merge_windows(most, p.nchunks);
     p.window = bfi::plan_negligible_window(precision, n_max);
     p.L = layout_for(p.nsub, p.nchunks, r.d, 2 + 3 * r.R, r.SL, r.TL);
 }
@@ -232,7 +241,7 @@ bfi_status launch_pass(bfi_server *s, int k, Pass &p, std::string &msg) {
               cuda(cudaMemcpyAsync(at(p.L.lo), p.lo.data(), sizeof(double) * p.nsub * r.d, cudaMemcpyHostToDevice, st), "copy") &&
               cuda(cudaMemcpyAsync(at(p.L.hi), p.hi.data(), sizeof(double) * p.nsub * r.d, cudaMemcpyHostToDevice, st), "copy") &&
               cuda(cudaMemcpyAsync(at(p.L.sid), p.sid.data(), sizeof(uint32_t) * p.nsub, cudaMemcpyHostToDevice, st), "copy") &&
-              cuda(cudaMemsetAsync(at(p.L.stats), 0, 4 * sizeof(unsigned long long), st), "memset");
+              cuda(cudaMemsetAsync(at(p.L.stats), 0, kCounters * sizeof(unsigned long long), st), "memset");
     int per_sm = 1;
     if (ok) ok = cuda(shape->occupancy[prec](r.lat.nx, r.lat.nt, &per_sm), "occupancy");
     const bfi::LatticeParams lp{r.lat.nx, r.lat.nt, r.lat.nu, r.lat.D, r.lat.a, r.lat.tau, r.lat.nonlinear, r.lat.mass2};
@@ -264,10 +273,12 @@ bfi_status launch_pass(bfi_server *s, int k, Pass &p, std::string &msg) {
         ok = false;
     }
     if (ok) {
-        const bfi::MergeArgs mg{lo, hi, static_cast<const int64_t *>(at(p.L.off)), static_cast<const double *>(at(p.L.part)),
-                                slots, p.nsub, r.R, r.d, 0, 0.0};
-        const bfi::TotalsArgs tg{slots, totals, static_cast<double *>(at(p.L.fbuf)), p.nsub, r.R};
-        ok = cuda(bfi::launch_merges(mg, tg, st), "merge launch") &&
+        const bfi::MergeArgs mg{lo, hi, static_cast<const uint64_t *>(at(p.L.smp)),
+                                static_cast<const int64_t *>(at(p.L.off)), static_cast<double *>(at(p.L.part)), slots,
+                                totals, static_cast<double *>(at(p.L.fbuf)),
+                                static_cast<unsigned long long *>(at(p.L.stats)) + 4, p.nsub, p.windows, r.R, r.d,
+                                1.0 / r.d, 0, 0.0};
+        ok = cuda(bfi::launch_merges(mg, st), "merge launch") &&
              cuda(cudaMemcpyAsync(sl.stage, slots, sizeof(double) * p.nsub * r.SL, cudaMemcpyDeviceToHost, st), "copy") &&
              cuda(cudaMemcpyAsync(sl.stage + static_cast<size_t>(p.nsub) * r.SL, totals, sizeof(double) * r.TL,
                                   cudaMemcpyDeviceToHost, st), "copy") &&

@@ -122,12 +122,16 @@ extern "C" bfi_status bfi_integrate_static_scratch(const bfi_lattice *lattice, i
     if (total >= (1ull << 62)) return bfi::set_error(BFI_E_INVALID, "total sample budget too large");
     const int R = lattice->nx / 2 + 1, K = 2 + 3 * R, d = lattice->nx * lattice->nt;
     const bfi::ChunkLayout layout = bfi::plan_chunk_layout(samples, nsub);
-    int64_t nchunks = 0;
-    for (int64_t s = 0; s < nsub; ++s) nchunks += layout.chunks_of(s, samples[s]);
+    int64_t nchunks = 0, most = 0;
+    for (int64_t s = 0; s < nsub; ++s) {
+        const int64_t c = layout.chunks_of(s, samples[s]);
+        nchunks += c;
+        most = c > most ? c : most;
+    }
     const size_t off_bytes = round_up(sizeof(int64_t) * (nsub + 1));
     const size_t smp_bytes = round_up(sizeof(uint64_t) * nsub);
     const size_t hint_bytes = round_up(sizeof(float) * nsub);
-    const size_t stat_bytes = round_up(2 * sizeof(unsigned long long));  // evaluated, next chunk
+    const size_t stat_bytes = round_up(3 * sizeof(unsigned long long));  // evaluated, next chunk, merge arrivals
     const size_t fbuf_bytes = round_up(sizeof(double) * 2 * nsub);
     const size_t par_bytes = round_up(sizeof(double) * static_cast<size_t>(nchunks > 0 ? nchunks : 1) * (K + 2));
     const size_t need = off_bytes + smp_bytes + hint_bytes + stat_bytes + fbuf_bytes + par_bytes;
@@ -159,12 +163,12 @@ extern "C" bfi_status bfi_integrate_static_scratch(const bfi_lattice *lattice, i
     int64_t grid = static_cast<int64_t>(sms) * (per_sm > 0 ? per_sm : 1);
     grid = grid < nchunks ? grid : (nchunks > 0 ? nchunks : 1);
 
-    // Everything below is ordered on 'stream'.  The two counters must start
+    // Everything below is ordered on 'stream'.  The counters must start
     // at zero; every other scratch word is written before it is read.
     cudaStream_t cs = static_cast<cudaStream_t>(stream);
     if ((e = cudaMemcpyAsync(d_samples, samples, sizeof(uint64_t) * nsub, cudaMemcpyHostToDevice, cs)) != cudaSuccess)
         return cuda_fail("copy of the budgets", e);
-    if ((e = cudaMemsetAsync(d_stats, 0, 2 * sizeof(unsigned long long), cs)) != cudaSuccess)
+    if ((e = cudaMemsetAsync(d_stats, 0, 3 * sizeof(unsigned long long), cs)) != cudaSuccess)
         return cuda_fail("clearing the counters", e);
     chunk_table<<<1, kScanThreads, 0, cs>>>(d_samples, nsub, layout, d_off);
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail("chunk table launch", e);
@@ -177,8 +181,8 @@ extern "C" bfi_status bfi_integrate_static_scratch(const bfi_lattice *lattice, i
         if ((e = shape->integrand[precision](a, lp, seed, job_id, static_cast<int>(grid), cs)) != cudaSuccess)
             return cuda_fail("integrand launch", e);
     }
-    const bfi::MergeArgs m{lo, hi, d_off, d_partials, slots, nsub, R, d, 0, 0.0};
-    const bfi::TotalsArgs t{slots, totals, d_fbuf, nsub, R};
-    if ((e = bfi::launch_merges(m, t, cs)) != cudaSuccess) return cuda_fail("merge launch", e);
+    const bfi::MergeArgs m{lo, hi, d_samples, d_off, d_partials, slots, totals, d_fbuf, d_stats + 2, nsub,
+                           bfi::merge_windows(most, nchunks), R, d, 1.0 / d, 0, 0.0};
+    if ((e = bfi::launch_merges(m, cs)) != cudaSuccess) return cuda_fail("merge launch", e);
     return BFI_OK;
 }
