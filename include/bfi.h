@@ -235,9 +235,10 @@ bfi_status bfi_plan_set_grid(bfi_plan *plan, int32_t ctas_per_sm);
 
 /* Samplers: how the unit point u (from Philox, see Conventions) becomes the
  * field v.  The box sampler (the default) takes v uniform in each box.  The
- * other two run in FP64 only (the FP32 screen's error bound does not hold
- * once a map stretches the coordinates, so every sample is evaluated in
- * FP64), on the warp-per-sample kernel:
+ * other two run in FP64 only.  TRANSFORM on a compiled shape leaves out
+ * negligible weights (see "Negligible weights") by an FP32 screen that bounds
+ * its own error for each sample; on other shapes, and with GAUSSIAN, every
+ * sample is evaluated in FP64:
  *
  *   BFI_SAMPLE_TRANSFORM  the infinite range mapped onto (-1, 1) (Sec. 4; the
  *       paper does not state its transform, this one is ours):
@@ -317,8 +318,9 @@ bfi_status bfi_plan_get_screen_stats(bfi_plan *plan, uint64_t *screened, int32_t
  *   full_screen  samples screened in one stage with the full FP32 action
  *                (samples = stage1 + full_screen for the box sampler)
  *   evaluated    samples fully evaluated (point, action, products, weight;
- *                for the TRANSFORM and GAUSSIAN samplers, which have no
- *                screen, every sample whose weight was computed)
+ *                for the TRANSFORM and GAUSSIAN samplers, whose stage1,
+ *                survivors and full_screen are 0, every sample whose weight
+ *                was computed)
  *   two_stage_shape  1 when the shape's kernels have the split compiled in
  *   rest_screen      1 when stage 2 adds the rest of the action to P (Nt = 2,
  *                    mass2 = 0), 0 when it screens survivors in full

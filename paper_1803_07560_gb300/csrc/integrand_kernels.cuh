@@ -561,21 +561,25 @@ struct SmemSums<double, K, BLOCK> {
 // error below 2^-42 of their magnitudes; only its partial and the butterfly
 // are double.  (In double the same took a multiply, an add and, per thread,
 // an exp on the FP64 pipe, 2 lanes per SM and clock, for every short chunk.)
-template <typename Real, int K, int R, int BLOCK>
+// With GIVEN the record's shift is *s_mb as the caller left it (behind a
+// barrier) instead.
+template <typename Real, int K, int R, int BLOCK, bool GIVEN = false>
 __device__ __forceinline__ void chunk_record(const SmemSums<Real, K, BLOCK> &acc, double m_t, double *s_f,
                                              double *s_mb, double *out, uint64_t cnt) {
     constexpr int WARPS = BLOCK / 32;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    s_f[tid] = m_t;
-    __syncthreads();
-    if (warp == 0) {
-        double mn = INFINITY;
-        for (int t = lane; t < BLOCK; t += 32) mn = fmin(mn, s_f[t]);
+    if constexpr (!GIVEN) {
+        s_f[tid] = m_t;
+        __syncthreads();
+        if (warp == 0) {
+            double mn = INFINITY;
+            for (int t = lane; t < BLOCK; t += 32) mn = fmin(mn, s_f[t]);
 #pragma unroll
-        for (int off = 16; off > 0; off >>= 1) mn = fmin(mn, __shfl_xor_sync(0xffffffffu, mn, off));
-        if (lane == 0) *s_mb = mn;
+            for (int off = 16; off > 0; off >>= 1) mn = fmin(mn, __shfl_xor_sync(0xffffffffu, mn, off));
+            if (lane == 0) *s_mb = mn;
+        }
+        __syncthreads();
     }
-    __syncthreads();
     const double mb = *s_mb;
     if constexpr (std::is_same<Real, float>::value) {
         const double n = (m_t - mb) * (1.0 / kLn2);  // >= 0; NaN or huge: no weight

@@ -12,13 +12,13 @@
 //                  unit point by the Box-Muller transform, S_eff = S(v) -
 //                  |z|^2 / 2 and weight 0 outside the box (d <= 40)
 //
-// There is no FP32 screen: the map stretches the coordinates without bound
-// near y = +-1, so no fixed margin covers the FP32 action's error there, and
-// inside a subvolume S_eff varies far less than it does over a box of the
-// plain field (most samples carry weight).  Every sample is evaluated in FP64;
-// the kernel is bound by GB300's FP64 pipe, so its FP64 work per sample is
-// kept small: one reciprocal per coordinate by Newton's iteration instead of
-// a division, and one logarithm per sample for all of ln J.
+// transform_f64 screens its samples in FP32 first, with a bound on the screen's
+// own error for each sample, and evaluates in FP64 those that may carry
+// weight (about one in twenty at 10x2 over all of R^20).  gaussian_f64
+// evaluates every sample: under its proposal nine in ten carry weight.  Both
+// are bound by GB300's FP64 pipe, so the FP64 work of an evaluation is kept
+// small: one reciprocal per coordinate by Newton's iteration instead of a
+// division, and one logarithm per sample for all of ln J.
 #pragma once
 
 #include "integrand_kernels.cuh"
@@ -61,82 +61,422 @@ struct LogProduct {
     }
 };
 
-// Compiled for one resident CTA per SM (all 255 registers a thread may
-// have): the FP64 pipe (two lanes per SM and clock) takes a warp instruction
-// every 64 cycles per scheduler, which two warps per scheduler keep busy, so
-// occupancy buys nothing and spilling the d FP64 coordinates would cost.
+// ---------------------------------------------------------------------------
+// FP32 screen of the range map, with bounds.  For a box inside [-1, 1]^d it
+// returns S_lo and S_hi around the S_eff that the FP64 evaluation computes
+// (u = 2^-24 below; "relative" errors are to first order):
+//   * 1 + y = (1 + lo) + W u and 1 - y = (1 - hi) + W (1 - u) are sums of
+//     non-negative terms, u from the word and 1 - u from its complement, so
+//     both have a small relative error (5 u) however close y is to +-1;
+//     r = 1 / ((1 + y)(1 - y)), v = y r: |dv| <= eps a, a = |v| + 1, with
+//     eps = 32 u, which also covers the rounding of y in the evaluation.
+//   * The residual R = v_next + v (c_adv (v_r - v_l) + k1) - c_dif (v_r + v_l)
+//     then has |dR| <= (2 eps + 8 u) T, T the sum of its terms' magnitudes with
+//     a for |v|; the bound used is E = 2^-17 T, 1.8 times that.
+//     S between inv sum max(0, |R| - E)^2 and inv sum (|R| + E)^2.
+//   * ln J, J = prod (1 + y^2) r^2, one logarithm per Philox block: 1e-3 and
+//     2^-15 of it cover the products' errors and lg2.approx's.
+// The interval is a few thousandths wide for samples that matter, and it
+// grows with the terms that cancel in a residual; an overflow gives S_lo =
+// inf (true actions beyond 1e38) or NaN, which no comparison rejects.
+// ---------------------------------------------------------------------------
+struct MapBox {
+    float p0, m0, w;  // 1 + lo, 1 - hi, hi - lo
+};
+
+__device__ __forceinline__ MapBox map_box(double lo, double hi) {
+    return MapBox{__double2float_rn(1.0 + lo), __double2float_rn(1.0 - hi), __double2float_rn(hi - lo)};
+}
+
+// The screen's premises: the box inside [-1, 1], and constants within float's
+// range (an action that overflows is then beyond any window).
+__device__ __forceinline__ bool map_box_screens(double lo, double hi) { return lo >= -1.0 && hi <= 1.0 && hi > lo; }
+__device__ __forceinline__ bool map_consts_screen(const LatticeConst<float> &c) {
+    return c.inv_2Dtau >= 1e-30f && c.inv_2Dtau <= 1e30f && fabsf(c.c_adv) <= 1e15f && fabsf(c.k1) <= 1e15f &&
+           fabsf(c.neg_c_dif) <= 1e15f && c.half_mass2 <= 1e15f;
+}
+
+__device__ __forceinline__ float rcp_approx(float x) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
+template <int NX, int NT>
+__device__ __forceinline__ void transform_screen(uint32_t x, const PhiloxPrefix *pre, const RoundKeys &rk,
+                                                 const MapBox *box, const LatticeConst<float> &c, float &S_lo,
+                                                 float &S_hi) {
+    constexpr int D = NX * NT, NQ = (D + 3) / 4;
+    float v[D];
+    float ln_j = 0.f;
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) {
+        const uint4 b = philox_from_prefix(x, pre[q], rk);
+        const uint32_t w4[4] = {b.x, b.y, b.z, b.w};
+        float jac = 1.f;
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+            const int j = 4 * q + t;
+            if (j < D) {
+                const MapBox bx = box[j];
+                const float u = fmaf(__uint2float_rn(w4[t]), 0x1p-32f, 0x1p-33f);
+                const float u1 = fmaf(__uint2float_rn(~w4[t]), 0x1p-32f, 0x1p-33f);
+                const float p = fmaf(u, bx.w, bx.p0), m = fmaf(u1, bx.w, bx.m0);
+                const float r = rcp_approx(p * m), y = 0.5f * (p - m);
+                v[j] = y * r;
+                jac *= fmaf(y, y, 1.f) * (r * r);
+            }
+        }
+        ln_j += __log2f(jac);
+    }
+    ln_j *= 0.69314718f;
+    const float a_adv = fabsf(c.c_adv), a_k1 = fabsf(c.k1), a_dif = fabsf(c.neg_c_dif);
+    float low = 0.f, high = 0.f;
+#pragma unroll
+    for (int m = 0; m < NX; ++m) {
+#pragma unroll
+        for (int l = 0; l < NT; ++l) {
+            const float here = v[m * NT + l], next = v[m * NT + (l + 1) % NT];
+            const float right = v[((m + 1) % NX) * NT + l], left = v[((m + NX - 1) % NX) * NT + l];
+            float R = fmaf(here, fmaf(c.c_adv, right - left, c.k1), next);
+            R = fmaf(c.neg_c_dif, right + left, R);
+            const float side = fabsf(right) + fabsf(left) + 2.f;
+            float T = fmaf(fabsf(here) + 1.f, fmaf(a_adv, side, a_k1), fabsf(next) + 1.f);
+            T = fmaf(a_dif, side, T);
+            const float over = fmaf(0x1p-17f, T, fabsf(R)), under = fmaxf(fmaf(-0x1p-17f, T, fabsf(R)), 0.f);
+            low = fmaf(under, under, low);
+            high = fmaf(over, over, high);
+        }
+    }
+    low *= c.inv_2Dtau;
+    high *= c.inv_2Dtau;
+    if (c.half_mass2 != 0.f) {
+        float s_lo = 0.f, s_hi = 0.f;
+#pragma unroll
+        for (int j = 0; j < D; ++j) {
+            const float a = fabsf(v[j]), e = fmaf(0x1p-18f, a, 0x1p-18f), under = fmaxf(a - e, 0.f), over = a + e;
+            s_lo = fmaf(under, under, s_lo);
+            s_hi = fmaf(over, over, s_hi);
+        }
+        low = fmaf(c.half_mass2, s_lo, low);
+        high = fmaf(c.half_mass2, s_hi, high);
+    }
+    S_lo = fmaf(low, 1.f - 0x1p-15f, -fmaf(ln_j, 1.f + 0x1p-15f, 1e-3f));
+    S_hi = fmaf(high, 1.f + 0x1p-15f, -fmaf(ln_j, 1.f - 0x1p-15f, -1e-3f));
+}
+
+// Floats and doubles as integers in the same order (NaN aside), for atomicMin.
+__device__ __forceinline__ int order_f32(float x) {
+    const int b = __float_as_int(x);
+    return b ^ ((b >> 31) & 0x7fffffff);
+}
+__device__ __forceinline__ float unorder_f32(int b) { return __int_as_float(b ^ ((b >> 31) & 0x7fffffff)); }
+__device__ __forceinline__ long long order_f64(double x) {
+    const long long b = __double_as_longlong(x);
+    return b ^ ((b >> 63) & 0x7fffffffffffffffll);
+}
+__device__ __forceinline__ double unorder_f64(long long b) {
+    return __longlong_as_double(b ^ ((b >> 63) & 0x7fffffffffffffffll));
+}
+
+// Reference action of a subvolume: the smallest S_hi among its first
+// hint_samples(n_s) samples, or +inf where the screen is not to be used (its
+// premises fail, or the interval of that sample is wider than kMapResolved, the
+// margin that moves a shift, as in slabs close to +-1): every sample of the
+// subvolume is then evaluated.  Measured on GB300 at nu = 6 (2^20 to 2^24
+// samples, intervals of 0.1 to 8): 10x2 20.4 ms at a limit of 0.05 against
+// 0.80 ms at 1, 4 and 16; 32x2 4.95 ms at 0.05, 4.75 at 4, 0.81 at 16.  One
+// CTA per subvolume.
+constexpr float kMapResolved = 16.f;
+
+template <int NX, int NT>
+__global__ void __launch_bounds__(kBlock) hint_transform(const IntegrandArgs args, const LatticeConst<float> lc,
+                                                         const RoundKeys rk) {
+    constexpr int D = NX * NT, NQ = (D + 3) / 4;
+    __shared__ int s_min, s_low, s_bad;
+    __shared__ MapBox s_map[D];
+    __shared__ PhiloxPrefix s_pre[NQ];
+    const int64_t s = blockIdx.x;
+    const int tid = threadIdx.x;
+    if (tid == 0) {
+        s_min = s_low = order_f32(INFINITY);
+        s_bad = map_consts_screen(lc) ? 0 : 1;
+    }
+    __syncthreads();
+    const uint32_t sid = args.sub_id ? args.sub_id[s] : static_cast<uint32_t>(s);
+    if (tid < NQ) s_pre[tid] = philox_prefix(tid, 0u, sid, rk);
+    if (tid < D) {
+        const double lo = args.lo[s * D + tid], hi = args.hi[s * D + tid];
+        s_map[tid] = map_box(lo, hi);
+        if (!map_box_screens(lo, hi)) s_bad = 1;
+    }
+    __syncthreads();
+    const uint32_t n = static_cast<uint32_t>(hint_samples(args.samples[s]));
+    float mn = INFINITY, ln = INFINITY;
+    for (uint32_t k = tid; k < n; k += kBlock) {
+        float lo, hi;
+        transform_screen<NX, NT>(k, s_pre, rk, s_map, lc, lo, hi);
+        mn = fminf(mn, hi);
+        ln = fminf(ln, lo);
+    }
+    atomicMin(&s_min, order_f32(mn));
+    atomicMin(&s_low, order_f32(ln));
+    __syncthreads();
+    if (tid == 0) {
+        const float best = unorder_f32(s_min);
+        args.hint[s] = s_bad || !(best - unorder_f32(s_low) <= kMapResolved) ? INFINITY : best;
+    }
+}
 
 // ---------------------------------------------------------------------------
-// One CTA processes chunk blockIdx.x, then the chunks next_chunk hands it; thread t
-// evaluates samples first + t, first + t + B, ... of the chunk.  The Philox
-// words, the point y = lo + (hi - lo) u (the FP64 point of the box sampler)
-// and 1 - y^2 = (1 - y)(1 + y) are those of the definition; v_j = y_j r_j
-// with r_j = 1 / (1 - y_j^2), and J_j = (1 + y_j^2) r_j^2 joins the running
-// product.  Each thread's shift starts above every action and drops to its
-// first sample's S_eff, then moves down only when beaten by more than
-// kRescaleMargin (as in the box kernels); the chunk record merges the
-// threads at the smallest shift.  A chunk with no finite S_eff records
-// m = +inf and zero sums.
+// One CTA processes chunk blockIdx.x, then the chunks next_chunk hands it;
+// thread t screens samples first + t, first + t + B, ... of the chunk.  Those
+// whose S_lo is within the negligible-weight window of the reference (the
+// hint, then the smallest action evaluated) go to the warp's queue and are
+// evaluated in FP64, 32 at a time: the Philox words, the point y = lo +
+// (hi - lo) u (the FP64 point of the box sampler) and 1 - y^2 = (1 - y)(1 + y)
+// are those of the definition; v_j = y_j r_j with r_j = 1 / (1 - y_j^2), and
+// J_j = (1 + y_j^2) r_j^2 joins the running product.
+//
+// The record's shift is defined by the samples alone, not by which of them
+// are evaluated or where: every thread's shift drops from +inf to its first
+// sample's S_eff and from then on only to a sample more than kRescaleMargin
+// below it, and the record has the smallest of the threads' shifts.  The
+// screen follows each thread's shift as an interval [m_lo, m_hi] with the
+// sample k_m that set it; a sample that may or may not have moved it leaves
+// the interval wide ('open') until one lies surely below both ends.  At the
+// chunk's end the threads whose interval reaches the smallest m_hi decide:
+// k_m is as a rule among the evaluated samples (the window is wider than the
+// margin), whose S_eff was kept, and is evaluated now where the whole chunk
+// lies outside the window of another chunk's reference; an open thread's
+// samples, rarely any, are gone through again in FP64 by the whole CTA.
+// A chunk with no finite S_eff records m = +inf and zero sums.
+//
+// Where the hint is +inf every sample goes through the queue, a warp's row at
+// once, so that lane l evaluates its own sample and its sums' shift is the
+// thread's shift.
+//
+// What bounds it: the FP64 pipe takes a warp instruction every 64 cycles per
+// scheduler, ~590 of them an evaluation, against ~1000 instructions of the
+// screen per row of 32 samples; two CTAs per SM let one's evaluations run
+// under the other's screen (lattices over 32 sites hold the FP64 field of an
+// evaluation in over 128 registers: one CTA).
+//
+// Measured on GB300 (whole pass, against the kernel that evaluated every
+// sample; nu = 1, [-1, 1]^d bisected): 10x2, 256 x 2^16 samples 19.55 ->
+// 1.67 ms; one volume of 2^22 samples at 4x2 5.83 -> 1.00 ms (a third of its
+// samples carry weight), at 8x4 10.8 -> 0.55 ms; 500 x 524 at 10x2 3.06 ->
+// 0.46 ms.
 // ---------------------------------------------------------------------------
 template <int NX, int NT, int BLOCK>
-__global__ void __launch_bounds__(BLOCK, 1) transform_f64(const IntegrandArgs args, const LatticeConst<double> lc,
-                                                          const RoundKeys rk) {
+__global__ void __launch_bounds__(BLOCK, NX *NT <= 32 ? 2 : 1)
+    transform_f64(const IntegrandArgs args, const LatticeConst<double> lc, const LatticeConst<float> lcf,
+                  const RoundKeys rk) {
     constexpr int D = NX * NT;
     constexpr int R = NX / 2 + 1;
     constexpr int K = sum_count(R);
     constexpr int NQ = (D + 3) / 4;
+    constexpr int WARPS = BLOCK / 32;
     __shared__ ChunkShared<BLOCK> sh;
-    __shared__ double s_lo[D], s_w[D];
+    __shared__ double s_lo[D], s_w[D], s_S[BLOCK];
+    __shared__ MapBox s_map[D];
     __shared__ PhiloxPrefix s_pre[NQ];
     __shared__ double s_sums[K * BLOCK];
-    const int tid = threadIdx.x;
+    __shared__ uint32_t s_queue[WARPS][kQueueCap], s_km[BLOCK], s_known[BLOCK], s_open[WARPS];
+    __shared__ long long s_shift;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const unsigned lt = (1u << lane) - 1u;
+    uint32_t *queue = s_queue[warp];
     SmemSums<double, K, BLOCK> acc{s_sums + tid};
+    constexpr uint32_t kNone = 0xffffffffu;  // no sample (offsets in a chunk are below 2^31)
 
     for (int64_t c = blockIdx.x; c < args.nchunks; c = next_chunk(args, c, &sh.next)) {
         const ChunkView v = chunk_view(args, c, D);
+        const float hint = args.hint[v.s];
+        const bool direct = !(hint < INFINITY);
         if (tid < D) {
             s_lo[tid] = v.lo[tid];
             s_w[tid] = v.hi[tid] - v.lo[tid];
+            s_map[tid] = map_box(v.lo[tid], v.hi[tid]);
         }
         chunk_prefixes<D>(v, rk, s_pre);
-        if (tid == 0) sh.evaluated = 0u;
+        if (tid == 0) {
+            sh.evaluated = 0u;
+            sh.min_bits = order_f32(hint);
+            s_shift = order_f64(INFINITY);
+        }
+        s_km[tid] = s_known[tid] = kNone;
         acc.zero();
         __syncthreads();
 
-        double m_acc = INFINITY;
+        double m_acc = INFINITY;                    // shift of this thread's sums
+        float m_ref = hint, m_lo = INFINITY, m_hi = INFINITY;
+        bool open = false;
         unsigned n_eval = 0;
-        for (uint64_t k = tid; k < v.cnt; k += BLOCK) {
-            const uint32_t x = static_cast<uint32_t>(v.first + k);
-            double u[D];
-            LogProduct jac;
-#pragma unroll
-            for (int q = 0; q < NQ; ++q) {
-                const uint4 b = philox_from_prefix(x, s_pre[q], rk);
-                const uint32_t w4[4] = {b.x, b.y, b.z, b.w};
-#pragma unroll
-                for (int t = 0; t < 4; ++t) {
-                    const int j = 4 * q + t;
-                    if (j < D) {
-                        const double y = Coord<double>::map(w4[t], s_lo[j], s_w[j]);
-                        const double r = recip_newton((1.0 - y) * (1.0 + y));
-                        u[j] = y * r;
-                        jac.mul(fma(y, y, 1.0) * r * r);
-                        if (j % 2 == 1 || j == D - 1) jac.renorm();
+        int count = 0;
+        const uint32_t cnt = static_cast<uint32_t>(v.cnt), xb = static_cast<uint32_t>(v.first);
+        const uint32_t nrows = (cnt + BLOCK - 1) / BLOCK;
+        uint32_t again = 0u, again_row = 0u;        // the open thread whose samples are gone through again
+        double again_m = INFINITY;
+        bool ask = false;                           // this thread decides and its k_m has not been evaluated
+        // rows 0 .. nrows - 1; then the samples left in the queues; then the k_m that decide but were outside the
+        // window; then, rarely, an open thread's samples
+        for (uint32_t row = 0;;) {
+            const uint32_t k = row * BLOCK + tid;
+            uint32_t k_eval = 0u;
+            bool evaluate = false;
+            if (row < nrows) {
+                bool cand = false;
+                if (k < cnt) {
+                    cand = true;
+                    if (!direct) {
+                        float lo, hi;
+                        transform_screen<NX, NT>(xb + k, s_pre, rk, s_map, lcf, lo, hi);
+                        cand = !(lo > __fadd_ru(m_ref, args.skip_window));
+                        const float slack = kRescaleMargin + 0x1p-20f * fabsf(m_lo);
+                        if (hi < m_lo - slack || (m_lo == INFINITY && hi < INFINITY)) {
+                            m_lo = lo;
+                            m_hi = hi;
+                            open = !(lo > -INFINITY);
+                            s_km[tid] = k;
+                        } else if (!(m_hi < INFINITY && lo >= m_hi - kRescaleMargin + 0x1p-20f * fabsf(m_hi))) {
+                            m_lo = lo < m_lo ? lo : (lo == lo ? m_lo : -INFINITY);
+                            open = true;
+                        }
                     }
                 }
+                count = enqueue(queue, count, cand, k, lt);
+                evaluate = count >= 32;
+                if (evaluate) k_eval = queue[lane];
+            } else if (row == nrows) {
+                if (direct) {  // fewer than a row: the lanes' own samples
+                    evaluate = lane < count;
+                    if (evaluate) k_eval = queue[lane];
+                } else {       // gathered in warp order and evaluated in as few warps as possible
+                    uint32_t *flat = &s_queue[0][0];
+                    const uint32_t mine = lane < count ? queue[lane] : 0u;
+                    if (lane == 0) sh.left[warp] = count;
+                    __syncthreads();
+                    int off = 0, total = 0;
+#pragma unroll
+                    for (int w = 0; w < WARPS; ++w) {
+                        const int c_w = sh.left[w];
+                        off += w < warp ? c_w : 0;
+                        total += c_w;
+                    }
+                    if (lane < count) flat[off + lane] = mine;
+                    __syncthreads();
+                    evaluate = tid < total;
+                    if (evaluate) k_eval = flat[tid];
+                }
+            } else if (row == nrows + 1) {
+                evaluate = ask;
+                if (ask) k_eval = s_km[tid];
+            } else {
+                k_eval = (again_row + tid) * BLOCK + again;
+                evaluate = again_row + tid < nrows && k_eval < cnt;
+                s_S[tid] = INFINITY;
             }
-            const double S = action<NX, NT, double>(u, lc) - jac.log_value();
-            double Q[R];
-            products<NX, NT, double>(u, Q);
-            if (S < m_acc - kRescaleMargin) {  // the first sample, then rarely
-                rescale<double, K, R, BLOCK>(acc, exp(S - m_acc));
-                m_acc = S;
+            if (evaluate) {
+                const uint32_t x = xb + k_eval;
+                double u[D];
+                LogProduct jac;
+#pragma unroll
+                for (int q = 0; q < NQ; ++q) {
+                    const uint4 b = philox_from_prefix(x, s_pre[q], rk);
+                    const uint32_t w4[4] = {b.x, b.y, b.z, b.w};
+#pragma unroll
+                    for (int t = 0; t < 4; ++t) {
+                        const int j = 4 * q + t;
+                        if (j < D) {
+                            const double y = Coord<double>::map(w4[t], s_lo[j], s_w[j]);
+                            const double r = recip_newton((1.0 - y) * (1.0 + y));
+                            u[j] = y * r;
+                            jac.mul(fma(y, y, 1.0) * r * r);
+                            if (j % 2 == 1 || j == D - 1) jac.renorm();
+                        }
+                    }
+                }
+                const double S = action<NX, NT, double>(u, lc) - jac.log_value();
+                if (row <= nrows) {
+                    m_ref = fminf(m_ref, __double2float_ru(S));
+                    const uint32_t owner = k_eval % BLOCK;
+                    if (!direct && s_km[owner] == k_eval) {  // one evaluation of each sample: no two threads write
+                        s_S[owner] = S;
+                        s_known[owner] = k_eval;
+                    }
+                    double Q[R];
+                    products<NX, NT, double>(u, Q);
+                    if (S < m_acc - kRescaleMargin) {  // the first sample, then rarely
+                        rescale<double, K, R, BLOCK>(acc, exp(S - m_acc));
+                        m_acc = S;
+                    }
+                    accumulate<double, K, R, BLOCK>(acc, exp(m_acc - S), Q);
+                    ++n_eval;
+                } else {
+                    s_S[tid] = S;
+                }
             }
-            accumulate<double, K, R, BLOCK>(acc, exp(m_acc - S), Q);
-            ++n_eval;
+            if (row < nrows) {
+                if (evaluate) {
+                    count = dequeue32(queue, count);
+                    m_ref = unorder_f32(__reduce_min_sync(0xffffffffu, order_f32(m_ref)));
+                }
+                if (++row % kShareRows == 0 && row < nrows) {
+                    atomicMin(&sh.min_bits, order_f32(m_ref));
+                    __syncthreads();
+                    m_ref = unorder_f32(sh.min_bits);
+                    __syncthreads();
+                }
+                continue;
+            }
+            if (direct) break;
+            if (row == nrows) {
+                if (tid == 0) sh.min_bits = order_f32(INFINITY);
+                __syncthreads();
+                atomicMin(&sh.min_bits, order_f32(m_hi));
+                __syncthreads();
+                const bool decides = static_cast<uint32_t>(tid) < cnt && m_lo <= unorder_f32(sh.min_bits);
+                const bool known = !open && s_known[tid] == s_km[tid];
+                if (decides && known) atomicMin(&s_shift, order_f64(s_S[tid]));
+                const unsigned unknown = __ballot_sync(0xffffffffu, decides && open);
+                if (lane == 0) s_open[warp] = unknown;
+                ask = decides && !open && !known;
+                row = __syncthreads_or(ask) ? nrows + 1 : nrows + 2;
+                again_row = nrows;  // none in hand yet
+                if (row == nrows + 1) continue;
+            } else if (row == nrows + 1) {
+                if (ask) atomicMin(&s_shift, order_f64(s_S[tid]));
+                row = nrows + 2;
+            } else {
+                again_row += BLOCK;
+                __syncthreads();
+                for (int i = 0; i < BLOCK; ++i)  // every thread follows the same rule
+                    if (s_S[i] < again_m - kRescaleMargin) again_m = s_S[i];
+            }
+            __syncthreads();
+            if (again_row >= nrows) {  // the thread in hand is done: take the next one
+                if (tid == 0 && again_m < INFINITY) s_shift = min(s_shift, order_f64(again_m));
+                int w = 0;
+                while (w < WARPS && s_open[w] == 0u) ++w;
+                if (w == WARPS) break;
+                again = w * 32 + __ffs(s_open[w]) - 1;
+                again_row = 0u;
+                again_m = INFINITY;
+                __syncthreads();
+                if (tid == 0) s_open[w] &= s_open[w] - 1u;
+                __syncthreads();
+            }
         }
         add_evaluated(args.stats, n_eval, &sh.evaluated);
-        chunk_record<double, K, R, BLOCK>(acc, m_acc, sh.f, &sh.mb, args.partials + c * (K + 2), v.cnt);
+        if (direct) {
+            chunk_record<double, K, R, BLOCK>(acc, m_acc, sh.f, &sh.mb, args.partials + c * (K + 2), v.cnt);
+        } else {
+            __syncthreads();
+            if (tid == 0) sh.mb = unorder_f64(s_shift);
+            __syncthreads();
+            chunk_record<double, K, R, BLOCK, true>(acc, m_acc, sh.f, &sh.mb, args.partials + c * (K + 2), v.cnt);
+        }
     }
 }
 
@@ -273,7 +613,11 @@ constexpr OccupancyQuery gaussian_occupancy_entry() {
 template <int NX, int NT>
 cudaError_t launch_transform(const IntegrandArgs &args, const LatticeParams &p, uint32_t seed, uint32_t job, int grid,
                              cudaStream_t st) {
-    transform_f64<NX, NT, kBlock><<<grid, kBlock, 0, st>>>(args, make_const<double>(p), make_round_keys(seed, job));
+    const RoundKeys rk = make_round_keys(seed, job);
+    hint_transform<NX, NT><<<static_cast<unsigned>(args.nsub), kBlock, 0, st>>>(args, make_const<float>(p), rk);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    transform_f64<NX, NT, kBlock><<<grid, kBlock, 0, st>>>(args, make_const<double>(p), make_const<float>(p), rk);
     return cudaGetLastError();
 }
 
