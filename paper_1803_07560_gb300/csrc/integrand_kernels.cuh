@@ -543,6 +543,7 @@ struct SmemSums<double, K, BLOCK> {
         for (int k = 0; k < K; ++k) b[k * BLOCK] = 0.0;
     }
     __device__ __forceinline__ void add(int k, double x) { b[k * BLOCK] += x; }
+    __device__ __forceinline__ void fma_add(int k, double x, double y) { b[k * BLOCK] = fma(x, y, b[k * BLOCK]); }
     __device__ __forceinline__ void scale(int k, double f) { b[k * BLOCK] *= f; }
     __device__ __forceinline__ double value(int k) const { return b[k * BLOCK]; }
 };
@@ -620,16 +621,16 @@ __device__ __forceinline__ void chunk_record(const SmemSums<Real, K, BLOCK> &acc
     __syncthreads();
 }
 
-template <typename Real, int K, int R, int BLOCK>
-__device__ __forceinline__ void accumulate(SmemSums<Real, K, BLOCK> &acc, Real w, const Real (&Q)[R]) {
+template <int K, int R, int BLOCK>
+__device__ __forceinline__ void accumulate(SmemSums<double, K, BLOCK> &acc, double w, const double (&Q)[R]) {
     acc.add(0, w);
-    acc.add(1, w * w);
+    acc.fma_add(1, w, w);
 #pragma unroll
     for (int r = 0; r < R; ++r) {
-        const Real wq = w * Q[r];
+        const double wq = w * Q[r];
         acc.add(2 + r, wq);
-        acc.add(2 + R + r, w * wq);
-        acc.add(2 + 2 * R + r, wq * wq);
+        acc.fma_add(2 + R + r, w, wq);
+        acc.fma_add(2 + 2 * R + r, wq, wq);
     }
 }
 
@@ -827,7 +828,7 @@ __global__ void __launch_bounds__(BLOCK, min_blocks<NX, NT>()) integrand_f64(con
                 m = S;
                 m_acc = m;
             }
-            accumulate<double, K, R, BLOCK>(acc, exp(m - S), Q);
+            accumulate<K, R, BLOCK>(acc, exp(m - S), Q);
             ++n_eval;
         };
         // m_ref changes only where the queue is evaluated (then made uniform

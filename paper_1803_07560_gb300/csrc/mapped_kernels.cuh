@@ -21,6 +21,7 @@
 // division, and one logarithm per sample for all of ln J.
 #pragma once
 
+#include "gauss_tables.h"
 #include "integrand_kernels.cuh"
 
 namespace bfi {
@@ -411,7 +412,7 @@ __global__ void __launch_bounds__(BLOCK, NX *NT <= 32 ? 2 : 1)
                         rescale<double, K, R, BLOCK>(acc, exp(S - m_acc));
                         m_acc = S;
                     }
-                    accumulate<double, K, R, BLOCK>(acc, exp(m_acc - S), Q);
+                    accumulate<K, R, BLOCK>(acc, exp(m_acc - S), Q);
                     ++n_eval;
                 } else {
                     s_S[tid] = S;
@@ -481,8 +482,108 @@ __global__ void __launch_bounds__(BLOCK, NX *NT <= 32 ? 2 : 1)
 }
 
 // ---------------------------------------------------------------------------
+// Box-Muller pairs from words, by tables and short Taylor polynomials.  CUDA's
+// log, sqrt and sincospi took over half of the Gaussian kernel's FP64
+// instructions (about 70 of them a pair, on a pipe of 2 lanes per SM and
+// clock); their arguments are one 33-bit number each, so a table by a few
+// leading bits leaves little for a polynomial: 36 a pair.
+//
+//   t = -2 ln u, u = (w + 1/2) 2^-32 = m 2^e, m in [3/4, 3/2): with c a 20-bit
+//     approximation of 1/m from the 7 leading bits, z = m c - 1 is exact,
+//     |z| <= 2^-8, and t = -2 e ln 2 + 2 ln c - 2 ln(1 + z), the last by its
+//     Taylor polynomial of degree 7 (remainder below 2^-58 z).  c = 1 next to
+//     m = 1, so t keeps its relative accuracy as u -> 1.
+//   r = sqrt(t): one Newton step for 1/sqrt(t) from the hardware's
+//     approximation (PTX rsqrt.approx.ftz.f64) and one for the root.
+//   cos, sin of 2 pi u: the angle is that of the nearest of 1024 points of the
+//     circle plus x, |x| <= pi/1024; Taylor polynomials of degree 5 and 4
+//     (remainders below 2^-61), then the angle sum.
+// Table entries are pairs (hi, lo): the small terms are summed first, so a
+// result carries about one rounding.  Measured against 113-bit arithmetic over
+// 2^21 pairs, near the ends of u1 and the axes among them, the error of z over
+// r in units of 2^-53: at most 2.77, rms 0.512; with CUDA's functions 2.77 and
+// 0.534.
+// ---------------------------------------------------------------------------
+// constant data of each translation unit that includes this file
+static __device__ const tables::Octant kOctant = tables::make_octant();
+static __device__ const tables::Logs kLogs = tables::make_logs();
+
+struct __align__(16) Quad {
+    double x, y, z, w;
+};
+
+struct GaussTables {
+    Quad log_c[128];         // (c, 2 ln c as hi, lo) of the intervals of m
+    double2 log_e[34];       // 2 k ln 2, k = -e
+    Quad circle[1024];       // (cos, sin, and their lower parts) of 2 pi j / 1024
+};
+
+// Filled by the CTA (at least 129 threads); the caller synchronises.
+__device__ __forceinline__ void fill_gauss_tables(GaussTables &t) {
+    const int i = threadIdx.x;
+    if (i < 128) t.log_c[i] = Quad{kLogs.c[i], kLogs.hi[i], kLogs.lo[i], 0.0};
+    if (i < 34) t.log_e[i] = make_double2(kLogs.k_hi[i], kLogs.k_lo[i]);
+    if (i <= 128) {
+        const double c = kOctant.c[i], s = kOctant.s[i], cl = kOctant.c_lo[i], sl = kOctant.s_lo[i];
+#pragma unroll
+        for (int o = 0; o < 8; ++o) {  // the first octant, the others by symmetry
+            if (i == (o % 2 == 0 ? 128 : 0)) continue;
+            const bool even = o % 2 == 0;
+            const double a = even ? c : s, b = even ? s : c, al = even ? cl : sl, bl = even ? sl : cl;
+            const int q = o / 2, j = even ? o * 128 + i : (o + 1) * 128 - i;
+            t.circle[j] = q == 0   ? Quad{a, b, al, bl}
+                          : q == 1 ? Quad{-b, a, -bl, al}
+                          : q == 2 ? Quad{-a, -b, -al, -bl}
+                                   : Quad{b, -a, bl, -al};
+        }
+    }
+}
+
+// z0 = r cos(2 pi u2), z1 = r sin(2 pi u2) and r^2 = -2 ln u1 = z0^2 + z1^2.
+__device__ __forceinline__ void box_muller_words(uint32_t w1, uint32_t w2, const GaussTables &tab, double &z0,
+                                                 double &z1, double &r2) {
+    const double u = unit_f64(w1);
+    const int hi = __double2hiint(u), d = hi - 0x3fe80000, e = d >> 20;
+    const Quad c = tab.log_c[(d >> 13) & 127];
+    const double2 l2 = tab.log_e[-e];
+    const double z = fma(__hiloint2double(hi - (e << 20), __double2loint(u)), c.x, -1.0);
+    double q = fma(z, -2.0 / 7.0, 1.0 / 3.0);
+    q = fma(z, q, -2.0 / 5.0);
+    q = fma(z, q, 0.5);
+    q = fma(z, q, -2.0 / 3.0);
+    q = fma(z, q, 1.0);
+    const double t = (l2.x + c.y) + fma(z, -2.0, fma(z * z, q, l2.y + c.z));
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(t));
+    double g = t * y, h = __hiloint2double(__double2hiint(y) - 0x00100000, __double2loint(y));  // y / 2
+    const double f = fma(-g, h, 0.5);
+    g = fma(g, f, g);
+    h = fma(h, f, h);
+    const double r = fma(fma(-g, g, t), h, g);
+    // angle: 1024 points of 2^22 words each; x = 2 pi 2^-32 (k + 1/2), k = w2 - nearest, made a double by its bits:
+    // 2^52 + 2^31 + k, less 2^52 + 2^31
+    const uint32_t j = (w2 + 0x200000u) >> 22;
+    const uint32_t k = (w2 - (j << 22)) ^ 0x80000000u;
+    const double x = fma(__hiloint2double(0x43300000, static_cast<int>(k)) - 4503601774854144.0, 1.4629180792671596e-9,
+                         0.5 * 1.4629180792671596e-9);
+    const Quad p = tab.circle[j & 1023u];
+    const double x2 = x * x;
+    const double sx = fma(x * x2, fma(x2, 1.0 / 120.0, -1.0 / 6.0), x), cx1 = x2 * fma(x2, 1.0 / 24.0, -0.5);
+    z0 = r * (p.x + fma(-p.y, sx, fma(p.x, cx1, p.z)));
+    z1 = r * (p.y + fma(p.x, sx, fma(p.y, cx1, p.w)));
+    r2 = t;
+}
+
+// x >= lo and x < hi by integers that order as the doubles do: no FP64
+// instruction.  Bounds that are zero take the key of -0, which both zeros
+// reach; NaN bounds admit nothing.
+__device__ __forceinline__ long long bound_key(double b) {
+    return b != b ? 0x7fffffffffffffffll : order_f64(b == 0.0 ? -0.0 : b);
+}
+
+// ---------------------------------------------------------------------------
 // Gaussian importance sampling, thread per sample (d <= kGaussThreadMaxD):
-// z_{2p}, z_{2p+1} = box_muller(u_{2p}, u_{2p+1}) for the unit point u (the
+// z_{2p}, z_{2p+1} by Box-Muller from u_{2p}, u_{2p+1} for the unit point u (the
 // box plays no part in drawing; for odd d the pair of z_{d-1} takes word d of
 // the last Philox block), v = mean + F z, S_eff = S(v) - |z|^2 / 2, and
 // weight 0 outside the box
@@ -493,6 +594,15 @@ __global__ void __launch_bounds__(BLOCK, NX *NT <= 32 ? 2 : 1)
 // triangular F (TRI, the proposal bfi_gaussian_proposal returns) column j
 // stops at row j.  Samples outside the box are counted in n and skip the
 // action; the kernel counts the evaluated (inside) samples in stats.
+//
+// What bounds it: the FP64 pipe, which takes a warp instruction every 64
+// cycles per scheduler; two warps per scheduler keep it busy, so the kernel is
+// compiled for one CTA per SM with all the registers a thread may have.  At
+// 10x2 about 860 FP64 instructions a sample: 360 for the ten pairs, 210 for
+// F z, 120 for the action, 111 for the products, the rest for the weight and
+// the sums (883 counted, the pipe 91% busy; 1300 before the tables, the sums
+// by FMA and the box test off the pipe).  Measured on GB300, 2^22 samples at
+// 10x2: 9.94 -> 6.72 ms.
 // ---------------------------------------------------------------------------
 constexpr int kGaussThreadMaxD = 40;
 
@@ -506,20 +616,24 @@ __global__ void __launch_bounds__(BLOCK, 1) gaussian_f64(const IntegrandArgs arg
     constexpr int NQ = (D + 3) / 4;
     static_assert(D <= kGaussThreadMaxD, "the thread-per-sample Gaussian kernel holds v in registers");
     __shared__ ChunkShared<BLOCK> sh;
+    __shared__ GaussTables s_tab;
     __shared__ double s_ft[D * D];  // s_ft[j D + r] = F[r][j]
-    __shared__ double s_mean[D], s_lo[D], s_hi[D];
+    __shared__ double s_mean[D];
+    __shared__ long long s_lo[D], s_hi[D];
     __shared__ PhiloxPrefix s_pre[NQ];
     __shared__ double s_sums[K * BLOCK];
     const int tid = threadIdx.x;
     SmemSums<double, K, BLOCK> acc{s_sums + tid};
+    fill_gauss_tables(s_tab);
     for (int k = tid; k < D * D; k += BLOCK) s_ft[(k % D) * D + k / D] = factor[k];
     for (int k = tid; k < D; k += BLOCK) s_mean[k] = mean ? mean[k] : 0.0;
 
     for (int64_t c = blockIdx.x; c < args.nchunks; c = next_chunk(args, c, &sh.next)) {
         const ChunkView v = chunk_view(args, c, D);
         if (tid < D) {
-            s_lo[tid] = v.lo[tid];
-            s_hi[tid] = v.hi[tid];
+            const double lo = v.lo[tid], hi = v.hi[tid];
+            s_lo[tid] = bound_key(hi != hi ? hi : lo);
+            s_hi[tid] = bound_key(hi);
         }
         chunk_prefixes<D>(v, rk, s_pre);
         if (tid == 0) sh.evaluated = 0u;
@@ -530,6 +644,10 @@ __global__ void __launch_bounds__(BLOCK, 1) gaussian_f64(const IntegrandArgs arg
         unsigned n_eval = 0;
         for (uint64_t k = tid; k < v.cnt; k += BLOCK) {
             const uint32_t x = static_cast<uint32_t>(v.first + k);
+            // F is read again for every sample: hidden from the compiler, which would otherwise carry as much of it
+            // as it can in registers and spill the rest
+            const double *ft = s_ft;
+            asm volatile("" : "+l"(ft));
             double u[D];
 #pragma unroll
             for (int r = 0; r < D; ++r) u[r] = s_mean[r];
@@ -542,16 +660,16 @@ __global__ void __launch_bounds__(BLOCK, 1) gaussian_f64(const IntegrandArgs arg
                 for (int t = 0; t < 4; t += 2) {
                     const int j = 4 * q + t;
                     if (j < D) {
-                        double zp[2];
-                        box_muller(unit_f64(w4[t]), unit_f64(w4[t + 1]), zp[0], zp[1]);
+                        double zp[2], r2;
+                        box_muller_words(w4[t], w4[t + 1], s_tab, zp[0], zp[1], r2);
+                        zz = j + 1 < D ? zz + r2 : fma(zp[0], zp[0], zz);
 #pragma unroll
                         for (int e = 0; e < 2; ++e) {
                             if (j + e < D) {
                                 const double z = zp[e];
-                                zz = fma(z, z, zz);
 #pragma unroll
                                 for (int r = 0; r < (TRI ? j + e + 1 : D); ++r)
-                                    u[r] = fma(s_ft[(j + e) * D + r], z, u[r]);
+                                    u[r] = fma(ft[(j + e) * D + r], z, u[r]);
                             }
                         }
                     }
@@ -559,7 +677,10 @@ __global__ void __launch_bounds__(BLOCK, 1) gaussian_f64(const IntegrandArgs arg
             }
             bool inside = true;
 #pragma unroll
-            for (int r = 0; r < D; ++r) inside = inside && u[r] >= s_lo[r] && u[r] < s_hi[r];
+            for (int r = 0; r < D; ++r) {
+                const long long key = order_f64(u[r]);
+                inside = inside && key >= s_lo[r] && key < s_hi[r];
+            }
             if (!inside) continue;  // weight 0
             const double S = action<NX, NT, double>(u, lc) - 0.5 * zz;
             double Q[R];
@@ -568,7 +689,7 @@ __global__ void __launch_bounds__(BLOCK, 1) gaussian_f64(const IntegrandArgs arg
                 rescale<double, K, R, BLOCK>(acc, exp(S - m_acc));
                 m_acc = S;
             }
-            accumulate<double, K, R, BLOCK>(acc, exp(m_acc - S), Q);
+            accumulate<K, R, BLOCK>(acc, exp(m_acc - S), Q);
             ++n_eval;
         }
         add_evaluated(args.stats, n_eval, &sh.evaluated);
