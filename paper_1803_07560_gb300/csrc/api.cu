@@ -153,7 +153,7 @@ struct bfi_plan {
     int64_t *d_chunk_off = nullptr;
     uint64_t *d_samples = nullptr;
     double *d_partials = nullptr;
-    float *d_hint = nullptr;
+    float *d_hint = nullptr;  // behind the counters: zeroed with them
     unsigned long long *d_stats = nullptr;  // evaluated, fully screened, stage 1, next chunk, merge arrivals
     double *d_fbuf = nullptr;
     float skip_window = 0.f;
@@ -180,7 +180,6 @@ bfi_status bfi_plan_destroy(bfi_plan *plan) {
         cudaFree(plan->d_chunk_off);
         cudaFree(plan->d_samples);
         cudaFree(plan->d_partials);
-        cudaFree(plan->d_hint);
         cudaFree(plan->d_stats);
         cudaFree(plan->d_fbuf);
         cudaFree(plan->d_map);
@@ -262,13 +261,14 @@ bfi_status bfi_plan_create(bfi_plan **out, const bfi_lattice *lattice, int64_t n
     const size_t hint_bytes = sizeof(float) * nsub;
     p->scratch_bytes = off_bytes + smp_bytes + par_bytes + hint_bytes + kPlanCounters * sizeof(unsigned long long) + sizeof(double) * 2 * nsub;
     if (cudaMalloc(&p->d_chunk_off, off_bytes) != cudaSuccess || cudaMalloc(&p->d_samples, smp_bytes) != cudaSuccess ||
-        cudaMalloc(&p->d_partials, par_bytes) != cudaSuccess || cudaMalloc(&p->d_hint, hint_bytes) != cudaSuccess ||
-        cudaMalloc(&p->d_stats, kPlanCounters * sizeof(unsigned long long)) != cudaSuccess ||
+        cudaMalloc(&p->d_partials, par_bytes) != cudaSuccess ||
+        cudaMalloc(&p->d_stats, kPlanCounters * sizeof(unsigned long long) + hint_bytes) != cudaSuccess ||
         cudaMalloc(&p->d_fbuf, sizeof(double) * 2 * nsub) != cudaSuccess) {
         cudaGetLastError();
         bfi_plan_destroy(p);
         return fail(BFI_E_NOMEM, "device allocation of %zu bytes failed", p->scratch_bytes);
     }
+    p->d_hint = reinterpret_cast<float *>(p->d_stats + kPlanCounters);
     e = cudaMemcpy(p->d_chunk_off, off.data(), off_bytes, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(p->d_samples, samples, smp_bytes, cudaMemcpyHostToDevice);
     if (e != cudaSuccess) {
@@ -326,7 +326,8 @@ bfi_status bfi_plan_execute(bfi_plan *plan, const double *lo, const double *hi, 
     if (g.err != cudaSuccess) return fail(BFI_E_CUDA, "cannot select device: %s", cudaGetErrorString(g.err));
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     if (plan->timing) BFI_CUDA(cudaEventRecord(plan->ev[0], st));
-    BFI_CUDA(cudaMemsetAsync(plan->d_stats, 0, kPlanCounters * sizeof(unsigned long long), st));
+    BFI_CUDA(cudaMemsetAsync(plan->d_stats, 0,
+                             kPlanCounters * sizeof(unsigned long long) + sizeof(float) * plan->nsub, st));
     if (plan->nchunks > 0) {
         bfi::IntegrandArgs a{lo,           hi,           sub_id,        plan->d_samples,     plan->d_chunk_off,
                              plan->d_partials, plan->d_hint, plan->d_stats, plan->nsub, plan->nchunks,

@@ -37,7 +37,8 @@ struct IntegrandArgs {
     const uint64_t *samples;   // [nsub]
     const int64_t *chunk_off;  // [nsub + 1]
     double *partials;          // [nchunks * (K + 2)]
-    float *hint;               // [nsub] reference actions written by hint_f32
+    float *hint;               // [nsub] zeroed per execution: reference actions (put_hint, get_hint; the range map's
+                               // kernels keep plain floats)
     unsigned long long *stats; // [1] fully evaluated samples (zeroed per execution), or null
     int64_t nsub;
     int64_t nchunks;

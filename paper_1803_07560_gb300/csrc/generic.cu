@@ -425,7 +425,7 @@ __global__ void __launch_bounds__(kGBlock, lane_min_blocks<SPL, NT>()) generic_i
             }
             __syncthreads();
         }
-        const float hint = args.hint[v.s];
+        const float hint = get_hint(args.hint, v.s);
         float m_ref = hint;
         double m_acc = static_cast<double>(hint);
         unsigned n_eval = 0;
@@ -687,7 +687,8 @@ __global__ void __launch_bounds__(kGBlock) generic_mapped(const GenArgs ga, cons
 }
 
 // Per-subvolume reference action: the smallest FP32 action among the first
-// hint_samples(n_s) samples.  One CTA per subvolume, warp per sample.
+// hint_samples(n_s) samples, warp per sample, gridDim.y CTAs per subvolume
+// (see hint_f32).
 __global__ void __launch_bounds__(kGBlock) generic_hint(const GenArgs ga) {
     extern __shared__ __align__(16) unsigned char sm[];
     const IntegrandArgs &args = ga.a;
@@ -695,6 +696,8 @@ __global__ void __launch_bounds__(kGBlock) generic_hint(const GenArgs ga) {
     const GenLayout &L = ga.L;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t s = blockIdx.x;
+    const uint64_t n = hint_samples(args.samples[s]);
+    if (blockIdx.y * kGWarps >= n) return;
     int *s_min = reinterpret_cast<int *>(sm + L.mw);
     build_next(sm, L, g);
     load_box(sm, L, g, args.lo + s * g.d, args.hi + s * g.d);
@@ -704,16 +707,15 @@ __global__ void __launch_bounds__(kGBlock) generic_hint(const GenArgs ga) {
     const float2 *bf = reinterpret_cast<const float2 *>(sm + L.box_f);
     float *uf = reinterpret_cast<float *>(sm + L.uf) + warp * g.dpad;
     const uint32_t sid = args.sub_id ? args.sub_id[s] : static_cast<uint32_t>(s);
-    const uint64_t n = hint_samples(args.samples[s]);
     float mn = INFINITY;
-    for (uint64_t k = warp; k < n; k += kGWarps) {
+    for (uint64_t k = blockIdx.y * kGWarps + warp; k < n; k += gridDim.y * kGWarps) {
         warp_point<float>(k, sid, ga.rk, g, [&](int j, uint32_t w) { return Coord<float>::map(w, bf[j].x, bf[j].y); }, uf);
         mn = fminf(mn, warp_action<float>(uf, next, g, ga.cf));
         __syncwarp();
     }
     if (lane == 0) atomicMin(s_min, __float_as_int(mn));
     __syncthreads();
-    if (threadIdx.x == 0) args.hint[s] = __int_as_float(*s_min);
+    if (threadIdx.x == 0) put_hint(args.hint, s, __int_as_float(*s_min));
 }
 
 // Action and products at given points, one warp per point.
@@ -771,7 +773,8 @@ cudaError_t gen_integrand_launcher(const IntegrandArgs &args, const LatticeParam
         e = cudaFuncSetAttribute(generic_integrand<FP64, SPL, NT, G>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  ga.L.total);
     if (e != cudaSuccess) return e;
-    generic_hint<<<static_cast<unsigned>(args.nsub), kGBlock, ga.L.total, st>>>(ga);
+    const dim3 hint_grid(static_cast<unsigned>(args.nsub), hint_splits(args.nsub, 16, 64));
+    generic_hint<<<hint_grid, kGBlock, ga.L.total, st>>>(ga);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     generic_integrand<FP64, SPL, NT, G><<<grid, kGBlock, ga.L.total, st>>>(ga);
     return cudaGetLastError();

@@ -67,15 +67,11 @@ template <typename At, typename Put>
 __device__ __forceinline__ double merge_list(int64_t count, int R, At at, Put put) {
     const int lane = threadIdx.x & 31, K = sum_count(R);
     // the smallest shift, by the integers that order as the doubles do (no shift is NaN): off the FP64 pipe
-    auto key = [](double x) {
-        const long long b = __double_as_longlong(x);
-        return b ^ ((b >> 63) & 0x7fffffffffffffffll);
-    };
-    long long lowest = key(INFINITY);
-    for (int64_t i = lane; i < count; i += 32) lowest = min(lowest, key(__ldcg(at(i) + 1)));
+    long long lowest = order_f64(INFINITY);
+    for (int64_t i = lane; i < count; i += 32) lowest = min(lowest, order_f64(__ldcg(at(i) + 1)));
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) lowest = min(lowest, __shfl_xor_sync(0xffffffffu, lowest, off));
-    const double m = __longlong_as_double(lowest ^ ((lowest >> 63) & 0x7fffffffffffffffll));
+    const double m = unorder_f64(lowest);
     for (int k0 = 0; k0 < K; k0 += 32) {
         const int k = k0 + lane;
         const bool mine = k < K, sq = mine && second_order(k, R);
@@ -85,7 +81,7 @@ __device__ __forceinline__ double merge_list(int64_t count, int R, At at, Put pu
             double f = 0.0, f2 = 0.0;  // of record c0 + lane; 0: no evaluated samples in it
             if (lane < cnt) {
                 const double mc = __ldcg(at(c0 + lane) + 1);
-                f = key(mc) == key(INFINITY) ? 0.0 : (key(mc) == lowest ? 1.0 : exp(m - mc));
+                f = order_f64(mc) == order_f64(INFINITY) ? 0.0 : (order_f64(mc) == lowest ? 1.0 : exp(m - mc));
                 f2 = f * f;
             }
             const unsigned weighted = __ballot_sync(0xffffffffu, __double_as_longlong(f) != 0);

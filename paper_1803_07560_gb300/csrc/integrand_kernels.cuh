@@ -72,6 +72,8 @@ struct BoxPair<double> {
     }
 };
 
+__device__ __forceinline__ float get_hint(const float *hint, int64_t s);
+
 // ---------------------------------------------------------------------------
 // Chunk set-up shared by the integrand kernels.
 // ---------------------------------------------------------------------------
@@ -110,44 +112,10 @@ __device__ __forceinline__ Real action(const Real (&u)[NX * NT], const LatticeCo
     return S;
 }
 
-// Raw Philox words of sample i: block q = (q, i lo, i hi, sid), word j%4.
-template <int D>
-__device__ __forceinline__ void sample_words(uint64_t i, uint32_t sid, const RoundKeys &rk, uint32_t (&w)[D]) {
-    constexpr int NQ = (D + 3) / 4;
-#pragma unroll
-    for (int q = 0; q < NQ; ++q) {
-        const uint4 b = philox4x32_10(
-            make_uint4(static_cast<uint32_t>(q), static_cast<uint32_t>(i), static_cast<uint32_t>(i >> 32), sid), rk);
-        const uint32_t w4[4] = {b.x, b.y, b.z, b.w};
-#pragma unroll
-        for (int t = 0; t < 4; ++t)
-            if (4 * q + t < D) w[4 * q + t] = w4[t];
-    }
-}
-
-// FP32 coordinates of sample i from the (lo, width) pairs in shared memory.
-template <int D>
-__device__ __forceinline__ void make_point_smem(uint64_t i, uint32_t sid, const RoundKeys &rk, const float2 *box,
-                                                float (&u)[D]) {
-    constexpr int NQ = (D + 3) / 4;
-#pragma unroll
-    for (int q = 0; q < NQ; ++q) {
-        const uint4 b = philox4x32_10(
-            make_uint4(static_cast<uint32_t>(q), static_cast<uint32_t>(i), static_cast<uint32_t>(i >> 32), sid), rk);
-        const uint32_t w4[4] = {b.x, b.y, b.z, b.w};
-#pragma unroll
-        for (int t = 0; t < 4; ++t) {
-            const int j = 4 * q + t;
-            if (j < D) {
-                const float2 bw = box[j];
-                u[j] = Coord<float>::map(w4[t], bw.x, bw.y);
-            }
-        }
-    }
-}
-
-// The same two from the chunk's Philox prefixes (one per block q, in shared
-// memory): x is the low word of the sample index.
+// The raw words of a sample, and its FP32 coordinates from the (lo, width)
+// pairs in shared memory, from the chunk's Philox prefixes (one per block q, in
+// shared memory): x is the low word of the sample index; block q holds words
+// 4 q to 4 q + 3.
 template <int D>
 __device__ __forceinline__ void sample_words_pre(uint32_t x, const PhiloxPrefix *pre, const RoundKeys &rk,
                                                  uint32_t (&w)[D]) {
@@ -493,6 +461,15 @@ constexpr int kShareRows = 128;
 constexpr float kMarginInv = 1.0f / 0.999f;  // the screen's 0.1% margin folded into its threshold
 constexpr float kRescaleMargin = 16.f;
 
+// Doubles as integers in the same order (NaN aside), off the FP64 pipe.
+__device__ __forceinline__ long long order_f64(double x) {
+    const long long b = __double_as_longlong(x);
+    return b ^ ((b >> 63) & 0x7fffffffffffffffll);
+}
+__device__ __forceinline__ double unorder_f64(long long b) {
+    return __longlong_as_double(b ^ ((b >> 63) & 0x7fffffffffffffffll));
+}
+
 __device__ __forceinline__ float warp_min(float x) {
     return __int_as_float(static_cast<int>(__reduce_min_sync(0xffffffffu, static_cast<unsigned>(__float_as_int(x)))));
 }
@@ -562,31 +539,43 @@ struct SmemSums<double, K, BLOCK> {
 // error below 2^-42 of their magnitudes; only its partial and the butterfly
 // are double.  (In double the same took a multiply, an add and, per thread,
 // an exp on the FP64 pipe, 2 lanes per SM and clock, for every short chunk.)
+// Sums of threads that evaluated nothing are zero, so warps of which no thread
+// evaluated any ('any' false throughout) are left out, which changes no bit: a
+// chunk of a few rows has its evaluations in one warp (the last candidates are
+// evaluated in as few as possible), and adding up the other seven's zeros took
+// longer than its screen.  The smallest shift is found by integers.
 // With GIVEN the record's shift is *s_mb as the caller left it (behind a
 // barrier) instead.
 template <typename Real, int K, int R, int BLOCK, bool GIVEN = false>
-__device__ __forceinline__ void chunk_record(const SmemSums<Real, K, BLOCK> &acc, double m_t, double *s_f,
-                                             double *s_mb, double *out, uint64_t cnt) {
+__device__ __forceinline__ void chunk_record(const SmemSums<Real, K, BLOCK> &acc, double m_t, bool any, double *s_f,
+                                             double *s_mb, int *s_any, double *out, uint64_t cnt) {
     constexpr int WARPS = BLOCK / 32;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const bool warp_any = __any_sync(0xffffffffu, any);
     if constexpr (!GIVEN) {
-        s_f[tid] = m_t;
-        __syncthreads();
-        if (warp == 0) {
-            double mn = INFINITY;
-            for (int t = lane; t < BLOCK; t += 32) mn = fmin(mn, s_f[t]);
+        // the warp's smallest shift into its first slot of s_f
+        long long mn = order_f64(m_t);
 #pragma unroll
-            for (int off = 16; off > 0; off >>= 1) mn = fmin(mn, __shfl_xor_sync(0xffffffffu, mn, off));
-            if (lane == 0) *s_mb = mn;
-        }
+        for (int off = 16; off > 0; off >>= 1) mn = min(mn, __shfl_xor_sync(0xffffffffu, mn, off));
+        __syncthreads();  // s_f holds the threads' shifts until here
+        if (lane == 0) s_f[warp] = unorder_f64(mn);
         __syncthreads();
+        if (tid == 0) {
+            mn = order_f64(s_f[0]);
+            for (int w = 1; w < WARPS; ++w) mn = min(mn, order_f64(s_f[w]));
+            *s_mb = unorder_f64(mn);
+        }
     }
+    if (lane == 0) s_any[warp] = warp_any;
+    __syncthreads();
     const double mb = *s_mb;
-    if constexpr (std::is_same<Real, float>::value) {
-        const double n = (m_t - mb) * (1.0 / kLn2);  // >= 0; NaN or huge: no weight
-        s_f[tid] = n < 1000.0 ? ldexp(1.0, -static_cast<int>(rint(n))) : 0.0;
-    } else {
-        s_f[tid] = (m_t == INFINITY) ? 0.0 : (m_t == mb ? 1.0 : exp(mb - m_t));
+    if (warp_any) {
+        if constexpr (std::is_same<Real, float>::value) {
+            const double n = (m_t - mb) * (1.0 / kLn2);  // >= 0; NaN or huge: no weight
+            s_f[tid] = n < 1000.0 ? ldexp(1.0, -static_cast<int>(rint(n))) : 0.0;
+        } else {
+            s_f[tid] = (m_t == INFINITY) ? 0.0 : (m_t == mb ? 1.0 : exp(mb - m_t));
+        }
     }
     __syncthreads();
     const Real *base = acc.b - tid;  // element k of thread t: sums of thread t
@@ -596,7 +585,10 @@ __device__ __forceinline__ void chunk_record(const SmemSums<Real, K, BLOCK> &acc
         if constexpr (std::is_same<Real, float>::value) {
             using F32Sums = SmemSums<float, K, BLOCK>;
             DF p{0.f, 0.f};
-            for (int t = lane; t < BLOCK; t += 32) {
+#pragma unroll 1  // unrolled, its loads in flight spilled the screen's registers
+            for (int w = 0; w < WARPS; ++w) {
+                if (!s_any[w]) continue;
+                const int t = w * 32 + lane;
                 const double f = s_f[t];
                 const float ff = static_cast<float>(sq ? f * f : f);
                 p = df_add_f(p, __fmul_rn(base[k * BLOCK + t], ff));
@@ -604,7 +596,10 @@ __device__ __forceinline__ void chunk_record(const SmemSums<Real, K, BLOCK> &acc
             }
             part = static_cast<double>(p.h) + static_cast<double>(p.l);
         } else {
-            for (int t = lane; t < BLOCK; t += 32) {
+#pragma unroll 2
+            for (int w = 0; w < WARPS; ++w) {
+                if (!s_any[w]) continue;
+                const int t = w * 32 + lane;
                 SmemSums<Real, K, BLOCK> other{const_cast<Real *>(base) + t};
                 const double f = s_f[t];
                 part = __dadd_rn(part, __dmul_rn(other.value(k), sq ? f * f : f));
@@ -666,7 +661,7 @@ struct ChunkShared {
     double f[BLOCK];  // per-thread shift factors of the chunk record
     double mb;
     long long next;   // the chunk this CTA takes next
-    int left[BLOCK / 32];  // each warp's candidates left at the end of the chunk
+    int left[BLOCK / 32];  // each warp's candidates left at the end of the chunk, then whether it evaluated any
     int min_bits;
     unsigned evaluated;
     unsigned screened;
@@ -794,7 +789,7 @@ __global__ void __launch_bounds__(BLOCK, min_blocks<NX, NT>()) integrand_f64(con
             s_box[tid] = make_float2(__fmaf_rn(-0.99999994f, w_f, lo_f), w_f);
         }
         chunk_prefixes<D>(v, rk, s_pre);
-        const float hint = args.hint[v.s];
+        const float hint = get_hint(args.hint, v.s);
         float m_ref = hint;
         // the thread's shift lives in its shared-memory slot (only evaluations touch it)
         double &m_acc = sh.f[tid];
@@ -937,7 +932,7 @@ __global__ void __launch_bounds__(BLOCK, min_blocks<NX, NT>()) integrand_f64(con
         add_evaluated(args.stats, n_eval, &sh.evaluated);
         if (PartialScreen<NX, NT>::enabled) add_screened(args.screened, n_full, &sh.screened);
         if (two_stage) add_stage1(args.stage1, v.cnt);
-        chunk_record<double, K, R, BLOCK>(acc, double(m_acc), sh.f, &sh.mb, args.partials + c * (K + 2), v.cnt);
+        chunk_record<double, K, R, BLOCK>(acc, double(m_acc), n_eval > 0, sh.f, &sh.mb, sh.left, args.partials + c * (K + 2), v.cnt);
     }
 }
 
@@ -987,7 +982,7 @@ __global__ void __launch_bounds__(BLOCK, min_blocks<NX, NT>()) integrand_f32(con
             s_scr[tid] = make_float2(__fmaf_rn(-0.99999994f, w_f, lo_f), w_f);
         }
         chunk_prefixes<D>(v, rk, s_pre);
-        const float hint = args.hint[v.s];
+        const float hint = get_hint(args.hint, v.s);
         float m_ref = hint;
         // the thread's shift (double) lives in its shared-memory slot: only evaluations touch it
         double &m_acc = sh.f[tid];
@@ -1105,39 +1100,58 @@ __global__ void __launch_bounds__(BLOCK, min_blocks<NX, NT>()) integrand_f32(con
         add_evaluated(args.stats, n_eval, &sh.evaluated);
         if (PartialScreen<NX, NT>::enabled) add_screened(args.screened, n_full, &sh.screened);
         if (two_stage) add_stage1(args.stage1, v.cnt);
-        chunk_record<float, K, R, BLOCK>(acc, double(m_acc), sh.f, &sh.mb, args.partials + c * (K + 2), v.cnt);
+        chunk_record<float, K, R, BLOCK>(acc, double(m_acc), n_eval > 0, sh.f, &sh.mb, sh.left, args.partials + c * (K + 2), v.cnt);
     }
 }
 
 // Per-subvolume hint: the smallest FP32 action among the subvolume's first
 // hint_samples(n_s) samples (n_s/32, at least 256 and at most 4096: a few
-// percent of the work at most).  One CTA per subvolume.
+// percent of the work at most).  hint_splits CTAs share a subvolume, so that
+// a job of few subvolumes does not wait for one CTA's serial sweep while the
+// other SMs idle; they meet in a maximum over keys that order as the actions
+// do backwards (actions are >= 0; the array starts zeroed, +inf), which no
+// order of arrival changes.  Measured on GB300: 37 subvolumes at 7x3, a CTA
+// each, 214 us; 14 us with 64 CTAs each (generic_hint).
 __host__ __device__ constexpr uint64_t hint_samples(uint64_t n) {
     return n < 256 ? n : (n / 32 < 256 ? 256 : (n / 32 > 4096 ? 4096 : n / 32));
+}
+// CTAs per subvolume that fill the device 'ctas_per_sm' deep, at most 'most'.
+inline unsigned hint_splits(int64_t nsub, int ctas_per_sm, int most) {
+    const int64_t want = static_cast<int64_t>(152) * ctas_per_sm / (nsub > 0 ? nsub : 1);
+    return static_cast<unsigned>(want < 1 ? 1 : (want > most ? most : want));
+}
+__device__ __forceinline__ void put_hint(float *hint, int64_t s, float action) {
+    atomicMax(reinterpret_cast<unsigned *>(hint) + s, 0x7f800000u - __float_as_uint(action));
+}
+__device__ __forceinline__ float get_hint(const float *hint, int64_t s) {
+    return __uint_as_float(0x7f800000u - __float_as_uint(hint[s]));
 }
 
 template <int NX, int NT>
 __global__ void __launch_bounds__(kBlock) hint_f32(const IntegrandArgs args, const LatticeConst<float> lc,
                                                    const RoundKeys rk) {
-    constexpr int D = NX * NT;
+    constexpr int D = NX * NT, NQ = (D + 3) / 4;
     __shared__ int s_min;
     __shared__ __align__(16) float2 s_box[D];
+    __shared__ PhiloxPrefix s_pre[NQ];
     const int64_t s = blockIdx.x;
+    const uint32_t n = static_cast<uint32_t>(hint_samples(args.samples[s]));
+    if (blockIdx.y * kBlock >= n) return;
+    const uint32_t sid = args.sub_id ? args.sub_id[s] : static_cast<uint32_t>(s);
     if (threadIdx.x == 0) s_min = __float_as_int(INFINITY);
+    if (threadIdx.x < NQ) s_pre[threadIdx.x] = philox_prefix(threadIdx.x, 0u, sid, rk);
     if (threadIdx.x < D) BoxPair<float>::load(args.lo + s * D, args.hi + s * D, threadIdx.x, s_box[threadIdx.x].x,
                                               s_box[threadIdx.x].y);
     __syncthreads();
-    const uint64_t n = hint_samples(args.samples[s]);
-    const uint32_t sid = args.sub_id ? args.sub_id[s] : static_cast<uint32_t>(s);
     float mn = INFINITY;
-    for (uint64_t k = threadIdx.x; k < n; k += blockDim.x) {
+    for (uint32_t k = blockIdx.y * kBlock + threadIdx.x; k < n; k += gridDim.y * kBlock) {
         float u[D];
-        make_point_smem<D>(k, sid, rk, s_box, u);
+        make_point_pre<D>(k, s_pre, rk, s_box, u);
         mn = fminf(mn, action<NX, NT, float>(u, lc));
     }
     atomicMin(&s_min, __float_as_int(mn));
     __syncthreads();
-    if (threadIdx.x == 0) args.hint[s] = __int_as_float(s_min);
+    if (threadIdx.x == 0) put_hint(args.hint, s, __int_as_float(s_min));
 }
 
 template <int NX, int NT, typename Real>
@@ -1194,7 +1208,8 @@ template <int NX, int NT, typename Real>
 cudaError_t launch_integrand(const IntegrandArgs &args, const LatticeParams &p, uint32_t seed, uint32_t job,
                              int grid, cudaStream_t st) {
     const RoundKeys rk = make_round_keys(seed, job);
-    hint_f32<NX, NT><<<static_cast<unsigned>(args.nsub), kBlock, 0, st>>>(args, make_const<float>(p), rk);
+    const dim3 hint_grid(static_cast<unsigned>(args.nsub), hint_splits(args.nsub, 8, 4096 / kBlock));
+    hint_f32<NX, NT><<<hint_grid, kBlock, 0, st>>>(args, make_const<float>(p), rk);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     if constexpr (sizeof(Real) == 8)

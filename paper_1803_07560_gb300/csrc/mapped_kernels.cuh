@@ -166,19 +166,12 @@ __device__ __forceinline__ void transform_screen(uint32_t x, const PhiloxPrefix 
     S_hi = fmaf(high, 1.f + 0x1p-15f, -fmaf(ln_j, 1.f - 0x1p-15f, -1e-3f));
 }
 
-// Floats and doubles as integers in the same order (NaN aside), for atomicMin.
+// Floats as integers in the same order (NaN aside), for atomicMin.
 __device__ __forceinline__ int order_f32(float x) {
     const int b = __float_as_int(x);
     return b ^ ((b >> 31) & 0x7fffffff);
 }
 __device__ __forceinline__ float unorder_f32(int b) { return __int_as_float(b ^ ((b >> 31) & 0x7fffffff)); }
-__device__ __forceinline__ long long order_f64(double x) {
-    const long long b = __double_as_longlong(x);
-    return b ^ ((b >> 63) & 0x7fffffffffffffffll);
-}
-__device__ __forceinline__ double unorder_f64(long long b) {
-    return __longlong_as_double(b ^ ((b >> 63) & 0x7fffffffffffffffll));
-}
 
 // Reference action of a subvolume: the smallest S_hi among its first
 // hint_samples(n_s) samples, or +inf where the screen is not to be used (its
@@ -471,12 +464,13 @@ __global__ void __launch_bounds__(BLOCK, NX *NT <= 32 ? 2 : 1)
         }
         add_evaluated(args.stats, n_eval, &sh.evaluated);
         if (direct) {
-            chunk_record<double, K, R, BLOCK>(acc, m_acc, sh.f, &sh.mb, args.partials + c * (K + 2), v.cnt);
+            chunk_record<double, K, R, BLOCK>(acc, m_acc, n_eval > 0, sh.f, &sh.mb, sh.left, args.partials + c * (K + 2), v.cnt);
         } else {
             __syncthreads();
             if (tid == 0) sh.mb = unorder_f64(s_shift);
             __syncthreads();
-            chunk_record<double, K, R, BLOCK, true>(acc, m_acc, sh.f, &sh.mb, args.partials + c * (K + 2), v.cnt);
+            chunk_record<double, K, R, BLOCK, true>(acc, m_acc, n_eval > 0, sh.f, &sh.mb, sh.left,
+                                                    args.partials + c * (K + 2), v.cnt);
         }
     }
 }
@@ -693,7 +687,7 @@ __global__ void __launch_bounds__(BLOCK, 1) gaussian_f64(const IntegrandArgs arg
             ++n_eval;
         }
         add_evaluated(args.stats, n_eval, &sh.evaluated);
-        chunk_record<double, K, R, BLOCK>(acc, m_acc, sh.f, &sh.mb, args.partials + c * (K + 2), v.cnt);
+        chunk_record<double, K, R, BLOCK>(acc, m_acc, n_eval > 0, sh.f, &sh.mb, sh.left, args.partials + c * (K + 2), v.cnt);
     }
 }
 

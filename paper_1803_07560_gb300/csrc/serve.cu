@@ -241,7 +241,7 @@ bfi_status launch_pass(bfi_server *s, int k, Pass &p, std::string &msg) {
               cuda(cudaMemcpyAsync(at(p.L.lo), p.lo.data(), sizeof(double) * p.nsub * r.d, cudaMemcpyHostToDevice, st), "copy") &&
               cuda(cudaMemcpyAsync(at(p.L.hi), p.hi.data(), sizeof(double) * p.nsub * r.d, cudaMemcpyHostToDevice, st), "copy") &&
               cuda(cudaMemcpyAsync(at(p.L.sid), p.sid.data(), sizeof(uint32_t) * p.nsub, cudaMemcpyHostToDevice, st), "copy") &&
-              cuda(cudaMemsetAsync(at(p.L.stats), 0, kCounters * sizeof(unsigned long long), st), "memset");
+              cuda(cudaMemsetAsync(at(p.L.hint), 0, p.L.stats - p.L.hint + kCounters * sizeof(unsigned long long), st), "memset");
     int per_sm = 1;
     if (ok) ok = cuda(shape->occupancy[prec](r.lat.nx, r.lat.nt, &per_sm), "occupancy");
     const bfi::LatticeParams lp{r.lat.nx, r.lat.nt, r.lat.nu, r.lat.D, r.lat.a, r.lat.tau, r.lat.nonlinear, r.lat.mass2};

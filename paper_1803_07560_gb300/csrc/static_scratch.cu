@@ -163,12 +163,12 @@ extern "C" bfi_status bfi_integrate_static_scratch(const bfi_lattice *lattice, i
     int64_t grid = static_cast<int64_t>(sms) * (per_sm > 0 ? per_sm : 1);
     grid = grid < nchunks ? grid : (nchunks > 0 ? nchunks : 1);
 
-    // Everything below is ordered on 'stream'.  The counters must start
+    // Everything below is ordered on 'stream'.  The hints and the counters behind them must start
     // at zero; every other scratch word is written before it is read.
     cudaStream_t cs = static_cast<cudaStream_t>(stream);
     if ((e = cudaMemcpyAsync(d_samples, samples, sizeof(uint64_t) * nsub, cudaMemcpyHostToDevice, cs)) != cudaSuccess)
         return cuda_fail("copy of the budgets", e);
-    if ((e = cudaMemsetAsync(d_stats, 0, 3 * sizeof(unsigned long long), cs)) != cudaSuccess)
+    if ((e = cudaMemsetAsync(d_hint, 0, hint_bytes + 3 * sizeof(unsigned long long), cs)) != cudaSuccess)
         return cuda_fail("clearing the counters", e);
     chunk_table<<<1, kScanThreads, 0, cs>>>(d_samples, nsub, layout, d_off);
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail("chunk table launch", e);
