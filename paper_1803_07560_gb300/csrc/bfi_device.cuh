@@ -68,16 +68,21 @@ __host__ __device__ __forceinline__ uint4 philox4x32_10(uint4 c, const RoundKeys
 // cross a multiple of 2^32) and sub_id s fixed.  In round 1 both products
 // (of q and of h) are then fixed, in round 2 the product of word 2, in round
 // 3 the product of word 0; philox_prefix folds those, with the round keys
-// they meet, into five words, and philox_from_prefix finishes from x with
-// 16 of the 20 products.  The result equals philox4x32_10((q, x, h, s)).
+// they meet, into four words a block.  Word 0 after round 1 is the same for
+// every block of a sample (x with philox_word0, fixed for the chunk), and so is
+// its product in round 2: philox_first takes it once, and philox_from_prefix
+// finishes each block with 15 more of the 20 products.  The result equals
+// philox4x32_10((q, x, h, s)).
+//
+// A 32x32->64-bit multiply takes GB300's heavy FMA pipe for four cycles a warp
+// instruction (an FFMA one, measured), and that pipe bounds the FP32 screen:
+// sharing the product is 2 of 48 multiplies of stage 1 at 10x2.
 // ---------------------------------------------------------------------------
 struct __align__(16) PhiloxPrefix {
-    uint32_t a;    // round 1: word 0 = a ^ x
     uint32_t g;    // round 2: word 2 = hi(M0 word0) ^ g
     uint32_t fk;   // round 3: word 0 = hi(M1 word2) ^ fk
     uint32_t h;    // round 3: word 2 = h ^ lo(M0 word0 of round 2)
     uint32_t l3;   // round 3: word 3
-    uint32_t pad[3];
 };
 
 __host__ __device__ __forceinline__ PhiloxPrefix philox_prefix(uint32_t q, uint32_t h, uint32_t s,
@@ -87,7 +92,6 @@ __host__ __device__ __forceinline__ PhiloxPrefix philox_prefix(uint32_t q, uint3
     // round 2: word 0 = hi(M1 w2) ^ w1 ^ k0 and word 1 = lo(M1 w2) are fixed
     const uint32_t e = mulhi32(kPhiloxM1, w2) ^ w1 ^ rk.k0[1], f = kPhiloxM1 * w2;
     PhiloxPrefix p;
-    p.a = mulhi32(kPhiloxM1, h) ^ rk.k0[0];
     p.g = w3 ^ rk.k1[1];
     // round 3: the product of word 0 (= e) is fixed
     p.fk = f ^ rk.k0[2];
@@ -96,10 +100,22 @@ __host__ __device__ __forceinline__ PhiloxPrefix philox_prefix(uint32_t q, uint3
     return p;
 }
 
-__host__ __device__ __forceinline__ uint4 philox_from_prefix(uint32_t x, const PhiloxPrefix &p, const RoundKeys &rk) {
-    const uint32_t c0 = p.a ^ x;                                   // round 1
-    const uint32_t c2 = mulhi32(kPhiloxM0, c0) ^ p.g, c3 = kPhiloxM0 * c0;   // round 2
-    const uint4 c = make_uint4(mulhi32(kPhiloxM1, c2) ^ p.fk, kPhiloxM1 * c2, p.h ^ c3, p.l3);  // round 3
+// Word 0 after round 1 is x ^ philox_word0(h).
+__host__ __device__ __forceinline__ uint32_t philox_word0(uint32_t h, const RoundKeys &rk) {
+    return mulhi32(kPhiloxM1, h) ^ rk.k0[0];
+}
+
+// The product of round 2 that the blocks of sample x share.
+struct PhiloxFirst {
+    uint32_t hi, lo;
+};
+__host__ __device__ __forceinline__ PhiloxFirst philox_first(uint32_t x, uint32_t word0) {
+    return PhiloxFirst{mulhi32(kPhiloxM0, x ^ word0), kPhiloxM0 * (x ^ word0)};
+}
+
+__host__ __device__ __forceinline__ uint4 philox_from_prefix(PhiloxFirst f, const PhiloxPrefix &p, const RoundKeys &rk) {
+    const uint32_t c2 = f.hi ^ p.g;                                                                   // round 2
+    const uint4 c = make_uint4(mulhi32(kPhiloxM1, c2) ^ p.fk, kPhiloxM1 * c2, p.h ^ f.lo, p.l3);  // round 3
     return philox_rounds(c, rk, 3);
 }
 

@@ -39,7 +39,7 @@ GenShape gen_shape(int nx, int nt) {
 
 // Dynamic shared memory layout of one CTA (byte offsets, 16-aligned).
 struct GenLayout {
-    int next, box_f, lo_d, w_d, uf, ud, sums, mw, pre4, pre1, fac, mean, zb, total;
+    int next, box_f, lo_d, w_d, uf, ud, sums, mw, pre, fac, mean, zb, total;
 };
 
 __host__ __device__ inline int align16(int x) { return (x + 15) & ~15; }
@@ -59,8 +59,7 @@ __host__ __device__ inline GenLayout gen_layout(const GenShape &g, int mapped = 
     L.ud = o;    o = align16(o + 8 * g.dpad * kGWarps);       // double point per warp
     L.sums = o;  o = align16(o + 8 * (g.K + g.R + 1) * kGWarps);  // per-warp sums (FP64, or FP32 sums + comps)
     L.mw = o;    o = align16(o + 8 * kGWarps + 16);            // per-warp shift, counter, next chunk
-    L.pre4 = o;  o = align16(o + 16 * g.nq);                   // Philox prefixes of the chunk (lane screen):
-    L.pre1 = o;  o = align16(o + 4 * g.nq);                    //   words a, g, fk, h as uint4, then l3
+    L.pre = o;   o = align16(o + 16 * g.nq);                   // Philox prefixes of the chunk (lane screen)
     L.fac = o;   if (gauss) o = align16(o + 8 * g.d * g.d);   // factor F, row-major
     L.mean = o;  if (gauss) o = align16(o + 8 * g.d);         // mean
     L.zb = o;    if (mapped) o = align16(o + 8 * g.dpad * kGWarps);  // per warp: y of the range map, or u then z
@@ -275,16 +274,15 @@ struct LaneScreen {
     __host__ __device__ static int prefix_slot(int q) { return (q % (C / 4)) * G + q / (C / 4); }
 
     // S of the group's own sample, whose index has low word i (the chunk's
-    // prefixes hold the rest), on every lane of the group.
-    __device__ __forceinline__ float action(uint32_t i, const uint4 *pre4, const uint32_t *pre1, const RoundKeys &rk,
+    // prefixes and word0 hold the rest), on every lane of the group.
+    __device__ __forceinline__ float action(uint32_t i, uint32_t word0, const PhiloxPrefix *pre, const RoundKeys &rk,
                                             const LatticeConst<float> &cf) const {
         const int lane = threadIdx.x & 31, t = lane & (G - 1), base = lane - t;
+        const PhiloxFirst first = philox_first(i, word0);
         float X[C];  // X[s NT + l]
 #pragma unroll
         for (int b = 0; b < C / 4; ++b) {
-            const uint4 a = pre4[b * G + t];
-            const PhiloxPrefix p{a.x, a.y, a.z, a.w, pre1[b * G + t], {0u, 0u, 0u}};
-            const uint4 r = philox_from_prefix(i, p, rk);
+            const uint4 r = philox_from_prefix(first, pre[b * G + t], rk);
             X[4 * b + 0] = Coord<float>::map(r.x, lo[4 * b + 0], w[4 * b + 0]);
             X[4 * b + 1] = Coord<float>::map(r.y, lo[4 * b + 1], w[4 * b + 1]);
             X[4 * b + 2] = Coord<float>::map(r.z, lo[4 * b + 2], w[4 * b + 2]);
@@ -413,16 +411,11 @@ __global__ void __launch_bounds__(kGBlock, lane_min_blocks<SPL, NT>()) generic_i
         typename ScreenOf<SPL, NT, G>::type scr;
         scr.load(bf);
         // the chunk's Philox prefixes: the sample index's high word and the sub_id are fixed within a chunk
-        uint4 *pre4 = reinterpret_cast<uint4 *>(sm + L.pre4);
-        uint32_t *pre1 = reinterpret_cast<uint32_t *>(sm + L.pre1);
+        PhiloxPrefix *pre = reinterpret_cast<PhiloxPrefix *>(sm + L.pre);
+        const uint32_t high = static_cast<uint32_t>(v.first >> 32), word0 = philox_word0(high, ga.rk);
         if constexpr (SPL > 0) {
-            for (int q = tid; q < g.nq; q += kGBlock) {
-                const PhiloxPrefix p = philox_prefix(static_cast<uint32_t>(q), static_cast<uint32_t>(v.first >> 32),
-                                                     v.sid, ga.rk);
-                const int at = decltype(scr)::prefix_slot(q);
-                pre4[at] = make_uint4(p.a, p.g, p.fk, p.h);
-                pre1[at] = p.l3;
-            }
+            for (int q = tid; q < g.nq; q += kGBlock)
+                pre[decltype(scr)::prefix_slot(q)] = philox_prefix(static_cast<uint32_t>(q), high, v.sid, ga.rk);
             __syncthreads();
         }
         const float hint = get_hint(args.hint, v.s);
@@ -435,7 +428,7 @@ __global__ void __launch_bounds__(kGBlock, lane_min_blocks<SPL, NT>()) generic_i
             // the screen of samples k0 .. k0 + P - 1 (group p of the warp screens k0 + p)
             float S_group;
             if constexpr (SPL > 0) {
-                S_group = scr.action(xb + k0 + (P > 1 ? lane / G : 0), pre4, pre1, ga.rk, ga.cf);
+                S_group = scr.action(xb + k0 + (P > 1 ? lane / G : 0), word0, pre, ga.rk, ga.cf);
             } else {
                 warp_point<float>(v.first + k0, v.sid, ga.rk, g, [&](int j, uint32_t w) { return Coord<float>::map(w, bf[j].x, bf[j].y); }, uf);
                 S_group = warp_action<float>(uf, next, g, ga.cf);

@@ -27,19 +27,27 @@
 
 namespace bfi {
 
-// Shared memory of integrand_f64 per CTA (the larger of the two kernels).
+// Shared memory of integrand_f64 per CTA, the larger of the two kernels: the
+// chunk's state, box and prefixes, the sums, three queues, and what the system
+// takes of every CTA.
 template <int NX, int NT>
 constexpr int integrand_smem_bytes() {
-    return 8 * (kBlock + 2) + 24 * NX * NT + 8 * (2 + 3 * (NX / 2 + 1)) * kBlock + 4 * (kBlock / 32) * 64;
+    return 9 * kBlock + 24 * NX * NT + 16 * ((NX * NT + 3) / 4 + 1) + 8 * (2 + 3 * (NX / 2 + 1)) * kBlock +
+           3 * 4 * (kBlock / 32) * 64 + 1024;
 }
 
-template <int NX, int NT>
+// By registers: 4 CTAs up to 32 sites, 3 to 48, 2 beyond; in FP64 no more than
+// shared memory holds, else the kernel would spill for CTAs that never run
+// (32x2: one CTA with all its registers; 2^27 samples 5.53 -> 5.13 ms on
+// GB300).  FP32 keeps to what FP64 can hold or 2.
+template <int NX, int NT, typename Real>
 constexpr int min_blocks() {
     constexpr int d = NX * NT;
     constexpr int by_regs = d <= 32 ? 4 : (d <= 48 ? 3 : 2);
     constexpr int by_smem = (227 * 1024) / integrand_smem_bytes<NX, NT>();
-    constexpr int b = by_regs < by_smem ? by_regs : by_smem;
-    return BFI_INTEGRAND_MIN_BLOCKS > 0 ? BFI_INTEGRAND_MIN_BLOCKS : (b > 0 ? b : 1);
+    constexpr int least = sizeof(Real) == 8 ? 1 : 2;
+    constexpr int b = by_regs < by_smem ? by_regs : (by_smem > least ? by_smem : least);
+    return BFI_INTEGRAND_MIN_BLOCKS > 0 ? BFI_INTEGRAND_MIN_BLOCKS : b;
 }
 
 
@@ -114,15 +122,16 @@ __device__ __forceinline__ Real action(const Real (&u)[NX * NT], const LatticeCo
 
 // The raw words of a sample, and its FP32 coordinates from the (lo, width)
 // pairs in shared memory, from the chunk's Philox prefixes (one per block q, in
-// shared memory): x is the low word of the sample index; block q holds words
-// 4 q to 4 q + 3.
+// shared memory, and behind them philox_word0 in the g of one more): x is the
+// low word of the sample index; block q holds words 4 q to 4 q + 3.
 template <int D>
 __device__ __forceinline__ void sample_words_pre(uint32_t x, const PhiloxPrefix *pre, const RoundKeys &rk,
                                                  uint32_t (&w)[D]) {
     constexpr int NQ = (D + 3) / 4;
+            const PhiloxFirst first = philox_first(x, pre[NQ].g);
 #pragma unroll
     for (int q = 0; q < NQ; ++q) {
-        const uint4 b = philox_from_prefix(x, pre[q], rk);
+        const uint4 b = philox_from_prefix(first, pre[q], rk);
         const uint32_t w4[4] = {b.x, b.y, b.z, b.w};
 #pragma unroll
         for (int t = 0; t < 4; ++t)
@@ -134,9 +143,10 @@ template <int D>
 __device__ __forceinline__ void make_point_pre(uint32_t x, const PhiloxPrefix *pre, const RoundKeys &rk,
                                                const float2 *box, float (&u)[D]) {
     constexpr int NQ = (D + 3) / 4;
+        const PhiloxFirst first = philox_first(x, pre[NQ].g);
 #pragma unroll
     for (int q = 0; q < NQ; ++q) {
-        const uint4 b = philox_from_prefix(x, pre[q], rk);
+        const uint4 b = philox_from_prefix(first, pre[q], rk);
         const uint32_t w4[4] = {b.x, b.y, b.z, b.w};
 #pragma unroll
         for (int t = 0; t < 4; ++t) {
@@ -149,12 +159,14 @@ __device__ __forceinline__ void make_point_pre(uint32_t x, const PhiloxPrefix *p
     }
 }
 
-// Prefixes of the chunk's blocks q = 0 .. NQ-1 (threads 0 .. NQ-1; the
+// Prefixes of the chunk's blocks q = 0 .. NQ-1 and word 0 (threads 0 .. NQ; the
 // caller synchronises before use).
 template <int D>
 __device__ __forceinline__ void chunk_prefixes(const ChunkView &v, const RoundKeys &rk, PhiloxPrefix *pre) {
     constexpr int NQ = (D + 3) / 4;
-    if (threadIdx.x < NQ) pre[threadIdx.x] = philox_prefix(threadIdx.x, static_cast<uint32_t>(v.first >> 32), v.sid, rk);
+    const uint32_t high = static_cast<uint32_t>(v.first >> 32);
+    if (threadIdx.x < NQ) pre[threadIdx.x] = philox_prefix(threadIdx.x, high, v.sid, rk);
+    if (threadIdx.x == NQ) pre[NQ].g = philox_word0(high, rk);
 }
 
 // ---------------------------------------------------------------------------
@@ -203,9 +215,10 @@ template <int NX, int NT, typename Map>
 __device__ __forceinline__ void make_pairs_pre(uint32_t x, const PhiloxPrefix *pre, const RoundKeys &rk,
                                                const float2 *box, Map map, float2 (&P)[(NX / 2) * NT]) {
     constexpr int D = NX * NT, NQ = (D + 3) / 4, H = NX / 2;
+    const PhiloxFirst first = philox_first(x, pre[NQ].g);
 #pragma unroll
     for (int q = 0; q < NQ; ++q) {
-        const uint4 b = philox_from_prefix(x, pre[q], rk);
+        const uint4 b = philox_from_prefix(first, pre[q], rk);
         const uint32_t w4[4] = {b.x, b.y, b.z, b.w};
 #pragma unroll
         for (int t = 0; t < 4; ++t) {
@@ -242,10 +255,11 @@ __device__ __forceinline__ float screen_action(uint32_t x, const PhiloxPrefix *p
         return action_pairs<NX, NT>(P, c);
     } else {
         constexpr int D = NX * NT, NQ = (D + 3) / 4;
+        const PhiloxFirst first = philox_first(x, pre[NQ].g);
         float u[D];
 #pragma unroll
         for (int q = 0; q < NQ; ++q) {
-            const uint4 b = philox_from_prefix(x, pre[q], rk);
+            const uint4 b = philox_from_prefix(first, pre[q], rk);
             const uint32_t w4[4] = {b.x, b.y, b.z, b.w};
 #pragma unroll
             for (int t = 0; t < 4; ++t)
@@ -309,10 +323,11 @@ __device__ __forceinline__ float partial_action(uint32_t x, const PhiloxPrefix *
         return 0.f;  // never called: the kernels take the one-stage path
     } else {
         constexpr int H = NT / 2;
+        const PhiloxFirst first = philox_first(x, pre[PS::NQ].g);
         float2 P[PS::MC * H];
 #pragma unroll
         for (int q = 0; q < PS::BP; ++q) {
-            const uint4 b = philox_from_prefix(x, pre[q], rk);
+            const uint4 b = philox_from_prefix(first, pre[q], rk);
             const uint32_t w4[4] = {b.x, b.y, b.z, b.w};
 #pragma unroll
             for (int t = 0; t < 4; ++t) {
@@ -366,11 +381,12 @@ __device__ __forceinline__ float rest_action(uint32_t x, const PhiloxPrefix *pre
     if constexpr (!RestScreen<NX, NT>::enabled) {
         return 0.f;  // never called: the kernels screen survivors in full
     } else {
+        const PhiloxFirst first = philox_first(x, pre[PS::NQ].g);
         float2 P[NX];  // P[m] = (u[m, 0], u[m, 1]); only the sites drawn here are read
 #pragma unroll
         for (int q = 0; q < PS::NQ; ++q) {
             if (q == 0 || q >= PS::BP - 1) {
-                const uint4 b = philox_from_prefix(x, pre[q], rk);
+                const uint4 b = philox_from_prefix(first, pre[q], rk);
                 P[2 * q] = make_float2(Map{}(b.x, box[4 * q]), Map{}(b.y, box[4 * q + 1]));
                 P[2 * q + 1] = make_float2(Map{}(b.z, box[4 * q + 2]), Map{}(b.w, box[4 * q + 3]));
             }
@@ -596,7 +612,7 @@ __device__ __forceinline__ void chunk_record(const SmemSums<Real, K, BLOCK> &acc
             }
             part = static_cast<double>(p.h) + static_cast<double>(p.l);
         } else {
-#pragma unroll 2
+#pragma unroll 1
             for (int w = 0; w < WARPS; ++w) {
                 if (!s_any[w]) continue;
                 const int t = w * 32 + lane;
@@ -756,7 +772,7 @@ __device__ __forceinline__ int dequeue32_pair(uint32_t *q, float *pq, int count)
 // sum_j |dS/dy_j| <= ~52 sqrt(2 d S) for unit parameters: 0.007 at 10x2).
 // ---------------------------------------------------------------------------
 template <int NX, int NT, int BLOCK>
-__global__ void __launch_bounds__(BLOCK, min_blocks<NX, NT>()) integrand_f64(const IntegrandArgs args,
+__global__ void __launch_bounds__(BLOCK, min_blocks<NX, NT, double>()) integrand_f64(const IntegrandArgs args,
                                                                                  const LatticeConst<double> lc,
                                                                                  const LatticeConst<float> lcf,
                                                                                  const RoundKeys rk) {
@@ -767,7 +783,7 @@ __global__ void __launch_bounds__(BLOCK, min_blocks<NX, NT>()) integrand_f64(con
     __shared__ ChunkShared<BLOCK> sh;
     __shared__ double s_lo[D], s_w[D];
     __shared__ __align__(16) float2 s_box[D];  // (lo', width) as floats for the FP32 screen (MapScreen)
-    __shared__ PhiloxPrefix s_pre[(D + 3) / 4];
+    __shared__ PhiloxPrefix s_pre[(D + 3) / 4 + 1];
     __shared__ double s_sums[K * BLOCK];
     __shared__ uint32_t s_queue[WARPS][kQueueCap];
     __shared__ uint32_t s_squeue[PartialScreen<NX, NT>::enabled ? WARPS : 1][kQueueCap];
@@ -949,7 +965,7 @@ __global__ void __launch_bounds__(BLOCK, min_blocks<NX, NT>()) integrand_f64(con
 // ---------------------------------------------------------------------------
 
 template <int NX, int NT, int BLOCK>
-__global__ void __launch_bounds__(BLOCK, min_blocks<NX, NT>()) integrand_f32(const IntegrandArgs args,
+__global__ void __launch_bounds__(BLOCK, min_blocks<NX, NT, float>()) integrand_f32(const IntegrandArgs args,
                                                                                  const LatticeConst<float> lc,
                                                                                  const LatticeConstDF lcd,
                                                                                  const RoundKeys rk) {
@@ -961,7 +977,7 @@ __global__ void __launch_bounds__(BLOCK, min_blocks<NX, NT>()) integrand_f32(con
     __shared__ ChunkShared<BLOCK> sh;
     __shared__ __align__(16) float2 s_box[D];  // (lo, width) as floats: the evaluation's exact points
     __shared__ __align__(16) float2 s_scr[D];  // (lo', width): the screen's points (MapScreen)
-    __shared__ PhiloxPrefix s_pre[(D + 3) / 4];
+    __shared__ PhiloxPrefix s_pre[(D + 3) / 4 + 1];
     __shared__ float s_sums[Sums::WORDS * BLOCK];
     __shared__ uint32_t s_queue[WARPS][kQueueCap];
     __shared__ uint32_t s_squeue[PartialScreen<NX, NT>::enabled ? WARPS : 1][kQueueCap];
@@ -1111,7 +1127,7 @@ __global__ void __launch_bounds__(BLOCK, min_blocks<NX, NT>()) integrand_f32(con
 // other SMs idle; they meet in a maximum over keys that order as the actions
 // do backwards (actions are >= 0; the array starts zeroed, +inf), which no
 // order of arrival changes.  Measured on GB300: 37 subvolumes at 7x3, a CTA
-// each, 214 us; 14 us with 64 CTAs each (generic_hint).
+// each, 214 us; 17 us with 64 CTAs each (generic_hint).
 __host__ __device__ constexpr uint64_t hint_samples(uint64_t n) {
     return n < 256 ? n : (n / 32 < 256 ? 256 : (n / 32 > 4096 ? 4096 : n / 32));
 }
@@ -1133,13 +1149,14 @@ __global__ void __launch_bounds__(kBlock) hint_f32(const IntegrandArgs args, con
     constexpr int D = NX * NT, NQ = (D + 3) / 4;
     __shared__ int s_min;
     __shared__ __align__(16) float2 s_box[D];
-    __shared__ PhiloxPrefix s_pre[NQ];
+    __shared__ PhiloxPrefix s_pre[NQ + 1];
     const int64_t s = blockIdx.x;
     const uint32_t n = static_cast<uint32_t>(hint_samples(args.samples[s]));
     if (blockIdx.y * kBlock >= n) return;
     const uint32_t sid = args.sub_id ? args.sub_id[s] : static_cast<uint32_t>(s);
     if (threadIdx.x == 0) s_min = __float_as_int(INFINITY);
     if (threadIdx.x < NQ) s_pre[threadIdx.x] = philox_prefix(threadIdx.x, 0u, sid, rk);
+    if (threadIdx.x == NQ) s_pre[NQ].g = philox_word0(0u, rk);
     if (threadIdx.x < D) BoxPair<float>::load(args.lo + s * D, args.hi + s * D, threadIdx.x, s_box[threadIdx.x].x,
                                               s_box[threadIdx.x].y);
     __syncthreads();

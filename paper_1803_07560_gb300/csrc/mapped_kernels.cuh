@@ -108,11 +108,12 @@ __device__ __forceinline__ void transform_screen(uint32_t x, const PhiloxPrefix 
                                                  const MapBox *box, const LatticeConst<float> &c, float &S_lo,
                                                  float &S_hi) {
     constexpr int D = NX * NT, NQ = (D + 3) / 4;
+    const PhiloxFirst first = philox_first(x, pre[NQ].g);
     float v[D];
     float ln_j = 0.f;
 #pragma unroll
     for (int q = 0; q < NQ; ++q) {
-        const uint4 b = philox_from_prefix(x, pre[q], rk);
+        const uint4 b = philox_from_prefix(first, pre[q], rk);
         const uint32_t w4[4] = {b.x, b.y, b.z, b.w};
         float jac = 1.f;
 #pragma unroll
@@ -189,7 +190,7 @@ __global__ void __launch_bounds__(kBlock) hint_transform(const IntegrandArgs arg
     constexpr int D = NX * NT, NQ = (D + 3) / 4;
     __shared__ int s_min, s_low, s_bad;
     __shared__ MapBox s_map[D];
-    __shared__ PhiloxPrefix s_pre[NQ];
+    __shared__ PhiloxPrefix s_pre[NQ + 1];
     const int64_t s = blockIdx.x;
     const int tid = threadIdx.x;
     if (tid == 0) {
@@ -199,6 +200,7 @@ __global__ void __launch_bounds__(kBlock) hint_transform(const IntegrandArgs arg
     __syncthreads();
     const uint32_t sid = args.sub_id ? args.sub_id[s] : static_cast<uint32_t>(s);
     if (tid < NQ) s_pre[tid] = philox_prefix(tid, 0u, sid, rk);
+    if (tid == NQ) s_pre[NQ].g = philox_word0(0u, rk);
     if (tid < D) {
         const double lo = args.lo[s * D + tid], hi = args.hi[s * D + tid];
         s_map[tid] = map_box(lo, hi);
@@ -274,7 +276,7 @@ __global__ void __launch_bounds__(BLOCK, NX *NT <= 32 ? 2 : 1)
     __shared__ ChunkShared<BLOCK> sh;
     __shared__ double s_lo[D], s_w[D], s_S[BLOCK];
     __shared__ MapBox s_map[D];
-    __shared__ PhiloxPrefix s_pre[NQ];
+    __shared__ PhiloxPrefix s_pre[NQ + 1];
     __shared__ double s_sums[K * BLOCK];
     __shared__ uint32_t s_queue[WARPS][kQueueCap], s_km[BLOCK], s_known[BLOCK], s_open[WARPS];
     __shared__ long long s_shift;
@@ -372,12 +374,12 @@ __global__ void __launch_bounds__(BLOCK, NX *NT <= 32 ? 2 : 1)
                 s_S[tid] = INFINITY;
             }
             if (evaluate) {
-                const uint32_t x = xb + k_eval;
+                const PhiloxFirst first = philox_first(xb + k_eval, s_pre[NQ].g);
                 double u[D];
                 LogProduct jac;
 #pragma unroll
                 for (int q = 0; q < NQ; ++q) {
-                    const uint4 b = philox_from_prefix(x, s_pre[q], rk);
+                    const uint4 b = philox_from_prefix(first, s_pre[q], rk);
                     const uint32_t w4[4] = {b.x, b.y, b.z, b.w};
 #pragma unroll
                     for (int t = 0; t < 4; ++t) {
@@ -614,7 +616,7 @@ __global__ void __launch_bounds__(BLOCK, 1) gaussian_f64(const IntegrandArgs arg
     __shared__ double s_ft[D * D];  // s_ft[j D + r] = F[r][j]
     __shared__ double s_mean[D];
     __shared__ long long s_lo[D], s_hi[D];
-    __shared__ PhiloxPrefix s_pre[NQ];
+    __shared__ PhiloxPrefix s_pre[NQ + 1];
     __shared__ double s_sums[K * BLOCK];
     const int tid = threadIdx.x;
     SmemSums<double, K, BLOCK> acc{s_sums + tid};
@@ -637,7 +639,7 @@ __global__ void __launch_bounds__(BLOCK, 1) gaussian_f64(const IntegrandArgs arg
         double m_acc = INFINITY;
         unsigned n_eval = 0;
         for (uint64_t k = tid; k < v.cnt; k += BLOCK) {
-            const uint32_t x = static_cast<uint32_t>(v.first + k);
+            const PhiloxFirst first = philox_first(static_cast<uint32_t>(v.first + k), s_pre[NQ].g);
             // F is read again for every sample: hidden from the compiler, which would otherwise carry as much of it
             // as it can in registers and spill the rest
             const double *ft = s_ft;
@@ -648,7 +650,7 @@ __global__ void __launch_bounds__(BLOCK, 1) gaussian_f64(const IntegrandArgs arg
             double zz = 0.0;
 #pragma unroll
             for (int q = 0; q < NQ; ++q) {
-                const uint4 b = philox_from_prefix(x, s_pre[q], rk);
+                const uint4 b = philox_from_prefix(first, s_pre[q], rk);
                 const uint32_t w4[4] = {b.x, b.y, b.z, b.w};
 #pragma unroll
                 for (int t = 0; t < 4; t += 2) {
