@@ -150,8 +150,10 @@ struct bfi_plan {
     int sms = 1, per_sm_max = 1, per_sm = 1;
     int R = 0, K = 0, d = 0;
     std::vector<uint64_t> samples;
+    unsigned char *block = nullptr;  // device memory of a plan that owns it (bfi_plan_create); a context's plan
+                                     // lies in the context's buffer
     int64_t *d_chunk_off = nullptr;
-    uint64_t *d_samples = nullptr;
+    uint64_t *d_samples = nullptr;   // behind the chunk table: one copy brings both
     double *d_partials = nullptr;
     float *d_hint = nullptr;  // behind the counters: zeroed with them
     unsigned long long *d_stats = nullptr;  // evaluated, fully screened, stage 1, next chunk, merge arrivals
@@ -166,6 +168,97 @@ struct bfi_plan {
     bool map_upper = false;   // Gaussian sampler: F is upper triangular
 };
 
+namespace {
+
+size_t round_up(size_t x) { return (x + 255) & ~size_t(255); }
+
+// Byte offsets of a plan's device memory: chunk table and budgets, counters
+// and hints (zeroed together), merge factors, chunk records.
+struct PlanBytes {
+    size_t tables, stats, fbuf, part, total;
+};
+PlanBytes plan_bytes(const bfi_plan &p) {
+    PlanBytes b;
+    size_t o = 0;
+    b.tables = o; o += round_up(sizeof(int64_t) * (2 * p.nsub + 1));
+    b.stats = o;  o += round_up(kPlanCounters * sizeof(unsigned long long) + sizeof(float) * p.nsub);
+    b.fbuf = o;   o += round_up(sizeof(double) * 2 * p.nsub);
+    b.part = o;   o += round_up(sizeof(double) * static_cast<size_t>(std::max<int64_t>(p.nchunks, 1)) * (p.K + 2));
+    b.total = o;
+    return b;
+}
+
+void plan_bind(bfi_plan &p, unsigned char *base, const PlanBytes &b) {
+    p.d_chunk_off = reinterpret_cast<int64_t *>(base + b.tables);
+    p.d_samples = reinterpret_cast<uint64_t *>(p.d_chunk_off + p.nsub + 1);
+    p.d_stats = reinterpret_cast<unsigned long long *>(base + b.stats);
+    p.d_hint = reinterpret_cast<float *>(p.d_stats + kPlanCounters);
+    p.d_fbuf = reinterpret_cast<double *>(base + b.fbuf);
+    p.d_partials = reinterpret_cast<double *>(base + b.part);
+}
+
+// Checks the job and fills everything of the plan but its device memory, with
+// the box sampler; 'tables' gets the chunk table and the budgets.  The device
+// is current.
+bfi_status plan_describe(bfi_plan *p, const bfi_lattice *lattice, int64_t nsub, const uint64_t *samples,
+                         bfi_precision precision, int device, std::vector<int64_t> &tables) {
+    if (precision != BFI_FP64 && precision != BFI_FP32) return fail(BFI_E_INVALID, "unknown precision %d", precision);
+    const bfi::ShapeKernels *shape = bfi::find_shape(lattice->nx, lattice->nt);
+    if (!shape)
+        return fail(BFI_E_UNSUPPORTED, "lattice %dx%d has no compiled kernel in this library", lattice->nx,
+                    lattice->nt);
+    uint64_t total = 0, n_max = 1;
+    for (int64_t s = 0; s < nsub; ++s) {
+        if (samples[s] >= (1ull << 48))
+            return fail(BFI_E_INVALID, "samples[%lld] = %llu must be < 2^48", static_cast<long long>(s),
+                        static_cast<unsigned long long>(samples[s]));
+        total += samples[s];
+        n_max = std::max<uint64_t>(n_max, samples[s]);
+    }
+    if (total >= (1ull << 62)) return fail(BFI_E_INVALID, "total sample budget too large");
+    p->device = device;
+    p->lat = to_params(lattice);
+    p->precision = precision;
+    p->shape = shape;
+    p->nsub = nsub;
+    p->R = num_r(lattice->nx);
+    p->K = bfi::sum_count(p->R);
+    p->d = lattice->nx * lattice->nt;
+    p->total = static_cast<int64_t>(total);
+    p->samples.assign(samples, samples + nsub);
+    p->layout = bfi::plan_chunk_layout(samples, nsub);
+    p->chunk_samples = p->layout.chunk_samples;
+    p->skip_window = negligible_window(precision, n_max);
+    p->sampler = BFI_SAMPLE_BOX;
+    p->log_norm = 0.0;
+    p->map_upper = false;
+    tables.assign(2 * nsub + 1, 0);
+    int64_t most = 0;
+    for (int64_t s = 0; s < nsub; ++s) {
+        const int64_t c = p->layout.chunks_of(s, samples[s]);
+        tables[s + 1] = tables[s] + c;
+        tables[nsub + 1 + s] = static_cast<int64_t>(samples[s]);
+        most = std::max(most, c);
+    }
+    p->nchunks = tables[nsub];
+    p->windows = bfi::merge_windows(most, p->nchunks);
+    int sms = 0, per_sm = 0;
+    cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
+    if (e == cudaSuccess) e = shape->occupancy[precision](lattice->nx, lattice->nt, &per_sm);
+    if (e != cudaSuccess) return fail(BFI_E_CUDA, "device query failed: %s", cudaGetErrorString(e));
+    p->sms = sms;
+    p->per_sm_max = per_sm > 0 ? per_sm : 1;
+    p->per_sm = p->per_sm_max;
+    const int64_t resident = static_cast<int64_t>(sms) * p->per_sm_max;
+    p->grid = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(p->nchunks, resident)));
+    p->scratch_bytes = sizeof(int64_t) * (nsub + 1) + sizeof(uint64_t) * nsub +
+                       sizeof(double) * static_cast<size_t>(std::max<int64_t>(p->nchunks, 1)) * (p->K + 2) +
+                       sizeof(float) * nsub + kPlanCounters * sizeof(unsigned long long) + sizeof(double) * 2 * nsub;
+    return BFI_OK;
+}
+
+}  // namespace
+
 extern "C" {
 
 int32_t bfi_num_r(int32_t nx) { return nx / 2 + 1; }
@@ -177,11 +270,7 @@ bfi_status bfi_plan_destroy(bfi_plan *plan) {
     if (!plan) return BFI_OK;
     {
         DeviceGuard g(plan->device);
-        cudaFree(plan->d_chunk_off);
-        cudaFree(plan->d_samples);
-        cudaFree(plan->d_partials);
-        cudaFree(plan->d_stats);
-        cudaFree(plan->d_fbuf);
+        cudaFree(plan->block);
         cudaFree(plan->d_map);
         for (auto &e : plan->ev)
             if (e) cudaEventDestroy(e);
@@ -199,78 +288,24 @@ bfi_status bfi_plan_create(bfi_plan **out, const bfi_lattice *lattice, int64_t n
     if (nsub < 1) return fail(BFI_E_INVALID, "nsub must be >= 1 (got %lld)", static_cast<long long>(nsub));
     if (!samples) return fail(BFI_E_INVALID, "samples is NULL");
     if (precision != BFI_FP64 && precision != BFI_FP32) return fail(BFI_E_INVALID, "unknown precision %d", precision);
-    const bfi::ShapeKernels *shape = bfi::find_shape(lattice->nx, lattice->nt);
-    if (!shape)
-        return fail(BFI_E_UNSUPPORTED, "lattice %dx%d has no compiled kernel in this library", lattice->nx,
-                    lattice->nt);
-    uint64_t total = 0;
-    for (int64_t s = 0; s < nsub; ++s) {
-        if (samples[s] >= (1ull << 48))
-            return fail(BFI_E_INVALID, "samples[%lld] = %llu must be < 2^48", static_cast<long long>(s),
-                        static_cast<unsigned long long>(samples[s]));
-        total += samples[s];
-    }
-    if (total >= (1ull << 62)) return fail(BFI_E_INVALID, "total sample budget too large");
-
     DeviceGuard g(device);
     if (g.err != cudaSuccess) return fail(BFI_E_CUDA, "cannot select device %d: %s", device, cudaGetErrorString(g.err));
-
     bfi_plan *p = new (std::nothrow) bfi_plan();
     if (!p) return fail(BFI_E_NOMEM, "host allocation failed");
-    p->device = device;
-    p->lat = to_params(lattice);
-    p->precision = precision;
-    p->shape = shape;
-    p->nsub = nsub;
-    p->R = num_r(lattice->nx);
-    p->K = bfi::sum_count(p->R);
-    p->d = lattice->nx * lattice->nt;
-    p->total = static_cast<int64_t>(total);
-    p->samples.assign(samples, samples + nsub);
-    p->layout = bfi::plan_chunk_layout(samples, nsub);
-    p->chunk_samples = p->layout.chunk_samples;
-    uint64_t n_max = 1;
-    for (int64_t s = 0; s < nsub; ++s) n_max = std::max<uint64_t>(n_max, samples[s]);
-    p->skip_window = negligible_window(precision, n_max);
-    std::vector<int64_t> off(nsub + 1, 0);
-    int64_t most = 0;
-    for (int64_t s = 0; s < nsub; ++s) {
-        const int64_t c = p->layout.chunks_of(s, samples[s]);
-        off[s + 1] = off[s] + c;
-        most = std::max(most, c);
-    }
-    p->nchunks = off[nsub];
-    p->windows = bfi::merge_windows(most, p->nchunks);
-
-    int sms = 0, per_sm = 0;
-    cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
-    if (e == cudaSuccess) e = shape->occupancy[precision](lattice->nx, lattice->nt, &per_sm);
-    if (e != cudaSuccess) {
+    std::vector<int64_t> tables;
+    if ((st = plan_describe(p, lattice, nsub, samples, precision, device, tables)) != BFI_OK) {
         delete p;
-        return fail(BFI_E_CUDA, "device query failed: %s", cudaGetErrorString(e));
+        return st;
     }
-    p->sms = sms;
-    p->per_sm_max = per_sm > 0 ? per_sm : 1;
-    p->per_sm = p->per_sm_max;
-    const int64_t resident = static_cast<int64_t>(sms) * p->per_sm_max;
-    p->grid = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(p->nchunks, resident)));
-
-    const size_t off_bytes = sizeof(int64_t) * (nsub + 1);
-    const size_t smp_bytes = sizeof(uint64_t) * nsub;
-    const size_t par_bytes = sizeof(double) * static_cast<size_t>(std::max<int64_t>(p->nchunks, 1)) * (p->K + 2);
-    const size_t hint_bytes = sizeof(float) * nsub;
-    p->scratch_bytes = off_bytes + smp_bytes + par_bytes + hint_bytes + kPlanCounters * sizeof(unsigned long long) + sizeof(double) * 2 * nsub;
-    if (cudaMalloc(&p->d_chunk_off, off_bytes) != cudaSuccess || cudaMalloc(&p->d_samples, smp_bytes) != cudaSuccess ||
-        cudaMalloc(&p->d_partials, par_bytes) != cudaSuccess ||
-        cudaMalloc(&p->d_stats, kPlanCounters * sizeof(unsigned long long) + hint_bytes) != cudaSuccess ||
-        cudaMalloc(&p->d_fbuf, sizeof(double) * 2 * nsub) != cudaSuccess) {
+    const PlanBytes b = plan_bytes(*p);
+    if (cudaMalloc(&p->block, b.total) != cudaSuccess) {
         cudaGetLastError();
+        p->block = nullptr;
         bfi_plan_destroy(p);
-        return fail(BFI_E_NOMEM, "device allocation of %zu bytes failed", p->scratch_bytes);
+        return fail(BFI_E_NOMEM, "device allocation of %zu bytes failed", b.total);
     }
-    p->d_hint = reinterpret_cast<float *>(p->d_stats + kPlanCounters);
-    e = cudaMemcpy(p->d_chunk_off, off.data(), off_bytes, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(p->d_samples, samples, smp_bytes, cudaMemcpyHostToDevice);
+    plan_bind(*p, p->block, b);
+    const cudaError_t e = cudaMemcpy(p->d_chunk_off, tables.data(), sizeof(int64_t) * tables.size(), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) {
         bfi_plan_destroy(p);
         return fail(BFI_E_CUDA, "copy of the chunk table failed: %s", cudaGetErrorString(e));
@@ -582,38 +617,68 @@ bfi_status bfi_plan_get_timing(bfi_plan *plan, float *ms) {
 }  // extern "C"
 
 // ---------------------------------------------------------------------------
-// Context: one device, one stream, a cached plan and device buffers.
+// Context: one device, one stream, a cached plan and one device buffer that
+// only grows, so that a caller whose jobs change from call to call (a round of
+// adaptive subdivision, a line of the line protocol) allocates nothing after
+// the largest.  A small job's chunk table and inputs go to the device in one
+// copy through page-locked memory, and its records and totals come back in
+// one; a copy from or to pageable memory waits in the driver.  Measured on
+// GB300 at 10x2: 3 subvolumes (1 KB up) 89 -> 78 us a call, 100 (35 KB) 100 ->
+// 92 us; adaptive subdivision at 4x2 over 9 rounds 1.19 -> 0.80 ms.  Larger jobs'
+// arrays are copied directly: 300 subvolumes (104 KB) take 119 us so, 117 us
+// through the buffer, 1000 take 215 us either way, and a caller's own
+// page-locked arrays would be copied once more.
 // ---------------------------------------------------------------------------
+constexpr size_t kStageBytes = size_t(64) << 10;
+
+// Byte offsets in the context's device buffer: what goes up (chunk table and
+// budgets, lo, hi, sub_id) and what comes down (slots, totals) lie together.
+struct CtxLayout {
+    PlanBytes plan;
+    size_t lo, hi, sid, up_end, slots, totals, total;
+};
+
 struct bfi_ctx {
     int device = 0;
     cudaStream_t stream = nullptr;
     std::atomic<bool> busy{false};
-    bfi_plan *plan = nullptr;
+    bfi_plan plan;                 // its device memory is in 'buf'
+    bool planned = false;          // plan and layout describe the last job, whose tables are on the device
+    CtxLayout at{};
     bfi_lattice lat{};
-    bfi_precision precision = BFI_FP64;
-    double *d_lo = nullptr, *d_hi = nullptr, *d_slots = nullptr, *d_totals = nullptr;
-    uint32_t *d_sid = nullptr;
-    size_t cap_lo = 0, cap_hi = 0, cap_sid = 0, cap_slots = 0, cap_totals = 0;
+    unsigned char *buf = nullptr;
+    size_t cap = 0;
+    unsigned char *stage = nullptr;  // page-locked, 2 kStageBytes: up, then down; null if it could not be had
     int32_t sampler = BFI_SAMPLE_BOX;         // applied to every plan the context makes
     std::vector<double> map_mean, map_factor;
+    std::vector<int64_t> tables;
 };
 
 namespace {
 
 bool same_lattice(const bfi_lattice &a, const bfi_lattice &b) { return std::memcmp(&a, &b, sizeof a) == 0; }
 
-template <typename T>
-bfi_status grow(T *&ptr, size_t &cap, size_t need) {
-    if (need <= cap) return BFI_OK;
-    cudaFree(ptr);
-    ptr = nullptr;
-    cap = 0;
-    if (cudaMalloc(&ptr, need * sizeof(T)) != cudaSuccess) {
-        cudaGetLastError();
-        return fail(BFI_E_NOMEM, "device allocation of %zu bytes failed", need * sizeof(T));
-    }
-    cap = need;
-    return BFI_OK;
+// The plan's own memory with the inputs behind the tables and the outputs at
+// the end.
+CtxLayout ctx_layout(const bfi_plan &p, const bfi_lattice &lat) {
+    CtxLayout L;
+    const size_t box = sizeof(double) * static_cast<size_t>(p.nsub) * p.d;
+    size_t o = sizeof(int64_t) * (2 * p.nsub + 1);
+    L.lo = o;     o += box;
+    L.hi = o;     o += box;
+    L.sid = o;    o += sizeof(uint32_t) * p.nsub;
+    L.up_end = o;
+    o = round_up(o);
+    L.plan = plan_bytes(p);
+    const size_t shift = o - round_up(sizeof(int64_t) * (2 * p.nsub + 1));
+    L.plan.stats += shift;
+    L.plan.fbuf += shift;
+    L.plan.part += shift;
+    o = L.plan.total + shift;
+    L.slots = o;  o += sizeof(double) * static_cast<size_t>(p.nsub) * bfi_slot_len(lat.nx);
+    L.totals = o; o += sizeof(double) * bfi_totals_len(lat.nx);
+    L.total = round_up(o);
+    return L;
 }
 
 struct BusyGuard {
@@ -645,6 +710,10 @@ bfi_status bfi_ctx_create(bfi_ctx **out, int device) {
         delete c;
         return fail(BFI_E_CUDA, "cudaStreamCreate failed: %s", cudaGetErrorString(e));
     }
+    if (cudaMallocHost(reinterpret_cast<void **>(&c->stage), 2 * kStageBytes) != cudaSuccess) {
+        cudaGetLastError();
+        c->stage = nullptr;
+    }
     *out = c;
     return BFI_OK;
 }
@@ -654,12 +723,9 @@ bfi_status bfi_ctx_destroy(bfi_ctx *ctx) {
     {
         DeviceGuard g(ctx->device);
         cudaStreamSynchronize(ctx->stream);
-        bfi_plan_destroy(ctx->plan);
-        cudaFree(ctx->d_lo);
-        cudaFree(ctx->d_hi);
-        cudaFree(ctx->d_sid);
-        cudaFree(ctx->d_slots);
-        cudaFree(ctx->d_totals);
+        cudaFree(ctx->buf);
+        cudaFree(ctx->plan.d_map);
+        cudaFreeHost(ctx->stage);
         cudaStreamDestroy(ctx->stream);
     }
     delete ctx;
@@ -682,9 +748,7 @@ bfi_status bfi_ctx_set_sampler(bfi_ctx *ctx, const bfi_sampler *sampler, int32_t
         if (sampler->mean) ctx->map_mean.assign(sampler->mean, sampler->mean + d);
     }
     ctx->sampler = kind;
-    // the next integration re-plans with the sampler
-    bfi_plan_destroy(ctx->plan);
-    ctx->plan = nullptr;
+    ctx->planned = false;  // the next integration re-plans with the sampler
     return BFI_OK;
 }
 
@@ -701,54 +765,97 @@ bfi_status bfi_integrate(bfi_ctx *ctx, const bfi_lattice *lattice, int64_t nsub,
     DeviceGuard g(ctx->device);
     if (g.err != cudaSuccess) return fail(BFI_E_CUDA, "cannot select device: %s", cudaGetErrorString(g.err));
 
-    bool replan = !ctx->plan || !same_lattice(ctx->lat, *lattice) || ctx->precision != precision ||
-                  ctx->plan->nsub != nsub ||
-                  std::memcmp(ctx->plan->samples.data(), samples, sizeof(uint64_t) * nsub) != 0;
+    const bool replan = !ctx->planned || !same_lattice(ctx->lat, *lattice) || ctx->plan.precision != precision ||
+                        ctx->plan.nsub != nsub ||
+                        std::memcmp(ctx->plan.samples.data(), samples, sizeof(uint64_t) * nsub) != 0;
+    bfi_plan *plan = &ctx->plan;
+    cudaStream_t s = ctx->stream;
     if (replan) {
-        bfi_plan_destroy(ctx->plan);
-        ctx->plan = nullptr;
-        st = bfi_plan_create(&ctx->plan, lattice, nsub, samples, precision, ctx->device);
-        if (st != BFI_OK) return st;
-        ctx->lat = *lattice;
-        ctx->precision = precision;
-        if (ctx->sampler != BFI_SAMPLE_BOX) {
-            const bool gauss = ctx->sampler == BFI_SAMPLE_GAUSSIAN;
-            if (gauss && ctx->map_factor.size() != static_cast<size_t>(ctx->plan->d) * ctx->plan->d) {
-                bfi_plan_destroy(ctx->plan);
-                ctx->plan = nullptr;
-                return fail(BFI_E_INVALID, "the context's Gaussian sampler was set for another dimension");
-            }
-            const bfi_sampler smp{ctx->sampler, gauss && !ctx->map_mean.empty() ? ctx->map_mean.data() : nullptr,
-                                  gauss ? ctx->map_factor.data() : nullptr};
-            st = bfi_plan_set_sampler(ctx->plan, &smp);
-            if (st != BFI_OK) {
-                bfi_plan_destroy(ctx->plan);
-                ctx->plan = nullptr;
-                return st;
+        ctx->planned = false;
+        if ((st = plan_describe(plan, lattice, nsub, samples, precision, ctx->device, ctx->tables)) != BFI_OK) return st;
+        ctx->at = ctx_layout(*plan, *lattice);
+        if (ctx->at.total > ctx->cap) {
+            // twice the last size at least, so that growing jobs do not allocate on every call
+            const size_t want = std::max(ctx->at.total, std::min(2 * ctx->cap, ctx->at.total + (size_t(256) << 20)));
+            cudaFree(ctx->buf);
+            ctx->buf = nullptr;
+            ctx->cap = 0;
+            if (cudaMalloc(&ctx->buf, want) == cudaSuccess) {
+                ctx->cap = want;
+            } else {
+                cudaGetLastError();
+                ctx->buf = nullptr;
+                if (cudaMalloc(&ctx->buf, ctx->at.total) != cudaSuccess) {
+                    cudaGetLastError();
+                    ctx->buf = nullptr;
+                    return fail(BFI_E_NOMEM, "device allocation of %zu bytes failed", ctx->at.total);
+                }
+                ctx->cap = ctx->at.total;
             }
         }
+        plan_bind(*plan, ctx->buf, ctx->at.plan);
+        ctx->lat = *lattice;
+        if (ctx->sampler != BFI_SAMPLE_BOX) {
+            const bool gauss = ctx->sampler == BFI_SAMPLE_GAUSSIAN;
+            if (gauss && ctx->map_factor.size() != static_cast<size_t>(plan->d) * plan->d)
+                return fail(BFI_E_INVALID, "the context's Gaussian sampler was set for another dimension");
+            const bfi_sampler smp{ctx->sampler, gauss && !ctx->map_mean.empty() ? ctx->map_mean.data() : nullptr,
+                                  gauss ? ctx->map_factor.data() : nullptr};
+            if (gauss) {  // the factor's memory is of its dimension
+                cudaFree(plan->d_map);
+                plan->d_map = nullptr;
+            }
+            if ((st = bfi_plan_set_sampler(plan, &smp)) != BFI_OK) return st;
+        }
     }
-    const int d = lattice->nx * lattice->nt;
-    const size_t nbox = static_cast<size_t>(nsub) * d;
-    const size_t nslot = static_cast<size_t>(nsub) * bfi_slot_len(lattice->nx);
-    if ((st = grow(ctx->d_lo, ctx->cap_lo, nbox)) != BFI_OK) return st;
-    if ((st = grow(ctx->d_hi, ctx->cap_hi, nbox)) != BFI_OK) return st;
-    if (sub_id && (st = grow(ctx->d_sid, ctx->cap_sid, static_cast<size_t>(nsub))) != BFI_OK) return st;
-    if ((st = grow(ctx->d_slots, ctx->cap_slots, nslot)) != BFI_OK) return st;
-    if ((st = grow(ctx->d_totals, ctx->cap_totals, static_cast<size_t>(bfi_totals_len(lattice->nx)))) != BFI_OK)
+    const CtxLayout &at = ctx->at;
+    unsigned char *buf = ctx->buf;
+    const size_t box = sizeof(double) * static_cast<size_t>(nsub) * plan->d, n_sid = sizeof(uint32_t) * nsub,
+                 n_slots = at.totals - at.slots, n_totals = sizeof(double) * bfi_totals_len(lattice->nx);
+    const size_t up = sub_id ? at.up_end : at.sid, from = replan ? 0 : at.lo;
+    const size_t down = slots ? n_slots + n_totals : n_totals;
+    const bool stage_up = ctx->stage && up <= kStageBytes, stage_down = ctx->stage && down <= kStageBytes;
+    unsigned char *h_up = ctx->stage, *h_down = ctx->stage + kStageBytes;
+    auto enqueue = [&]() -> bfi_status {
+        if (stage_up) {
+            if (replan) std::memcpy(h_up, ctx->tables.data(), sizeof(int64_t) * ctx->tables.size());
+            std::memcpy(h_up + at.lo, lo, box);
+            std::memcpy(h_up + at.hi, hi, box);
+            if (sub_id) std::memcpy(h_up + at.sid, sub_id, n_sid);
+            BFI_CUDA(cudaMemcpyAsync(buf + from, h_up + from, up - from, cudaMemcpyHostToDevice, s));
+        } else {
+            if (replan)
+                BFI_CUDA(cudaMemcpyAsync(buf, ctx->tables.data(), sizeof(int64_t) * ctx->tables.size(),
+                                         cudaMemcpyHostToDevice, s));
+            BFI_CUDA(cudaMemcpyAsync(buf + at.lo, lo, box, cudaMemcpyHostToDevice, s));
+            BFI_CUDA(cudaMemcpyAsync(buf + at.hi, hi, box, cudaMemcpyHostToDevice, s));
+            if (sub_id) BFI_CUDA(cudaMemcpyAsync(buf + at.sid, sub_id, n_sid, cudaMemcpyHostToDevice, s));
+        }
+        const bfi_status e = bfi_plan_execute(plan, reinterpret_cast<double *>(buf + at.lo),
+                                              reinterpret_cast<double *>(buf + at.hi),
+                                              sub_id ? reinterpret_cast<uint32_t *>(buf + at.sid) : nullptr, seed, job_id,
+                                              reinterpret_cast<double *>(buf + at.slots),
+                                              reinterpret_cast<double *>(buf + at.totals), s);
+        if (e != BFI_OK) return e;
+        if (stage_down) {
+            BFI_CUDA(cudaMemcpyAsync(h_down, buf + (slots ? at.slots : at.totals), down, cudaMemcpyDeviceToHost, s));
+        } else {
+            if (slots) BFI_CUDA(cudaMemcpyAsync(slots, buf + at.slots, n_slots, cudaMemcpyDeviceToHost, s));
+            BFI_CUDA(cudaMemcpyAsync(totals, buf + at.totals, n_totals, cudaMemcpyDeviceToHost, s));
+        }
+        BFI_CUDA(cudaStreamSynchronize(s));
+        return BFI_OK;
+    };
+    ctx->planned = false;
+    if ((st = enqueue()) != BFI_OK) {
+        cudaStreamSynchronize(s);  // nothing still reads the staging buffer or the caller's arrays
         return st;
-
-    cudaStream_t s = ctx->stream;
-    BFI_CUDA(cudaMemcpyAsync(ctx->d_lo, lo, nbox * sizeof(double), cudaMemcpyHostToDevice, s));
-    BFI_CUDA(cudaMemcpyAsync(ctx->d_hi, hi, nbox * sizeof(double), cudaMemcpyHostToDevice, s));
-    if (sub_id) BFI_CUDA(cudaMemcpyAsync(ctx->d_sid, sub_id, nsub * sizeof(uint32_t), cudaMemcpyHostToDevice, s));
-    st = bfi_plan_execute(ctx->plan, ctx->d_lo, ctx->d_hi, sub_id ? ctx->d_sid : nullptr, seed, job_id, ctx->d_slots,
-                          ctx->d_totals, s);
-    if (st != BFI_OK) return st;
-    if (slots) BFI_CUDA(cudaMemcpyAsync(slots, ctx->d_slots, nslot * sizeof(double), cudaMemcpyDeviceToHost, s));
-    BFI_CUDA(cudaMemcpyAsync(totals, ctx->d_totals, bfi_totals_len(lattice->nx) * sizeof(double),
-                             cudaMemcpyDeviceToHost, s));
-    BFI_CUDA(cudaStreamSynchronize(s));
+    }
+    ctx->planned = true;
+    if (stage_down) {
+        if (slots) std::memcpy(slots, h_down, n_slots);
+        std::memcpy(totals, h_down + (slots ? n_slots : 0), n_totals);
+    }
     return BFI_OK;
 }
 
