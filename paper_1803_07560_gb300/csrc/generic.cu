@@ -22,7 +22,8 @@ constexpr int kGWarps = kGBlock / 32;
 
 struct GenShape {
     int nx, nt, d, R, K, nq;
-    int dpad;  // per-warp stride of the point buffers: d rounded up to 4 (vector stores stay aligned)
+    int dpad;  // stride of a point in the buffers: d rounded up to 4 (vector stores stay aligned)
+    int batch; // float points a warp draws at once (draw_points)
 };
 
 GenShape gen_shape(int nx, int nt) {
@@ -34,6 +35,7 @@ GenShape gen_shape(int nx, int nt) {
     g.K = 2 + 3 * g.R;
     g.nq = (g.d + 3) / 4;
     g.dpad = 4 * g.nq;
+    g.batch = g.nq <= 16 ? 32 / g.nq : 1;
     return g;
 }
 
@@ -55,7 +57,7 @@ __host__ __device__ inline GenLayout gen_layout(const GenShape &g, int mapped = 
     L.box_f = o; o = align16(o + 8 * g.d);                    // float2 (lo, width)
     L.lo_d = o;  o = align16(o + 8 * g.d);                    // double lo
     L.w_d = o;   o = align16(o + 8 * g.d);                    // double width
-    L.uf = o;    o = align16(o + 4 * g.dpad * kGWarps);       // float point per warp
+    L.uf = o;    o = align16(o + 4 * g.dpad * g.batch * kGWarps);  // float points per warp
     L.ud = o;    o = align16(o + 8 * g.dpad * kGWarps);       // double point per warp
     L.sums = o;  o = align16(o + 8 * (g.K + g.R + 1) * kGWarps);  // per-warp sums (FP64, or FP32 sums + comps)
     L.mw = o;    o = align16(o + 8 * kGWarps + 16);            // per-warp shift, counter, next chunk
@@ -192,6 +194,34 @@ __device__ __forceinline__ void warp_point(uint64_t i, uint32_t sid, const Round
         } else {
             const uint32_t w4[4] = {b.x, b.y, b.z, b.w};
             for (int t = 0; t < 4 && j + t < nd; ++t) u[j + t] = box(j + t, w4[t]);
+        }
+    }
+    __syncwarp();
+}
+
+// The float points of samples first, first + step, ... (up to g.batch of them,
+// those below first + limit) into u, u + dpad, ...: a lane draws one Philox block,
+// so a lattice of nq <= 16 blocks would leave most lanes of a warp idle through
+// the ten rounds if it drew one sample at a time (nq = 6 at 7x3: 6 of 32).
+// p_of, q_of = lane / nq and lane % nq.  Measured on GB300, 64 subvolumes of
+// 50,001 samples in FP64: 5x3 827 -> 461 us a pass, 7x3 749 -> 470, 8x8 810 ->
+// 649; at 20x4 (20 blocks) one sample nearly fills the warp, and a test for the
+// batch in the same kernel cost 1 to 5%, so it is a kernel of its own.
+__device__ __forceinline__ void draw_points(uint64_t first, uint64_t step, uint64_t limit, uint32_t sid,
+                                            const RoundKeys &rk, const GenShape &g, const float2 *bf, int p_of, int q_of,
+                                            float *u) {
+    if (p_of < g.batch && p_of * step < limit) {
+        const uint64_t i = first + p_of * step;
+        const uint4 b = philox4x32_10(
+            make_uint4(static_cast<uint32_t>(q_of), static_cast<uint32_t>(i), static_cast<uint32_t>(i >> 32), sid), rk);
+        const int j = 4 * q_of;
+        float *at = u + p_of * g.dpad + j;
+        auto box = [&](int t, uint32_t w) { return Coord<float>::map(w, bf[j + t].x, bf[j + t].y); };
+        if (j + 4 <= g.d) {
+            store4(at, box(0, b.x), box(1, b.y), box(2, b.z), box(3, b.w));
+        } else {
+            const uint32_t w4[4] = {b.x, b.y, b.z, b.w};
+            for (int t = 0; j + t < g.d; ++t) at[t] = box(t, w4[t]);
         }
     }
     __syncwarp();
@@ -367,7 +397,8 @@ struct ScreenOf<0, NT, G> {
 // screen and evaluation with the compensated action near the minimum.  SPL > 0
 // takes the register-resident screen (Nx = G SPL, NT time slices; with G = 16
 // a warp screens two consecutive samples at once and evaluates the candidates
-// among them in sample order); SPL = 0 the shared-memory one, for any shape.
+// among them in sample order); SPL = 0 the shared-memory one, for any shape, with
+// NT = 1 drawing g.batch points at once (d <= 64).
 // ---------------------------------------------------------------------------
 // 16 coordinates a lane at SPL >= 2 (64x8, 128x4, 256x2, 512x1) compile to 96
 // registers without spilling when asked for 5 CTAs per SM (4 otherwise); 32x16
@@ -379,6 +410,7 @@ constexpr int lane_min_blocks() { return SPL * NT == 16 && SPL >= 2 ? 5 : 0; }
 template <bool FP64, int SPL, int NT, int G = 32>
 __global__ void __launch_bounds__(kGBlock, lane_min_blocks<SPL, NT>()) generic_integrand(const GenArgs ga) {
     constexpr int P = SPL > 0 ? 32 / G : 1;  // samples a warp screens at once
+    constexpr int kBatch = SPL == 0 && NT == 1;  // points drawn several at once (draw_points)
     extern __shared__ __align__(16) unsigned char sm[];
     const IntegrandArgs &args = ga.a;
     const GenShape &g = ga.g;
@@ -388,7 +420,8 @@ __global__ void __launch_bounds__(kGBlock, lane_min_blocks<SPL, NT>()) generic_i
     const float2 *bf = reinterpret_cast<const float2 *>(sm + L.box_f);
     const double *ld = reinterpret_cast<const double *>(sm + L.lo_d);
     const double *wd = reinterpret_cast<const double *>(sm + L.w_d);
-    float *uf = reinterpret_cast<float *>(sm + L.uf) + warp * g.dpad;
+    float *uf = reinterpret_cast<float *>(sm + L.uf) + warp * g.dpad * g.batch;
+    float *const uf_all = uf;
     double *ud = reinterpret_cast<double *>(sm + L.ud) + warp * g.dpad;
     double *mw = reinterpret_cast<double *>(sm + L.mw);
     unsigned *cnt_all = reinterpret_cast<unsigned *>(mw + kGWarps);
@@ -397,6 +430,7 @@ __global__ void __launch_bounds__(kGBlock, lane_min_blocks<SPL, NT>()) generic_i
     double *sd = reinterpret_cast<double *>(sm + L.sums) + warp * (g.K + g.R + 1);
     float *sf = reinterpret_cast<float *>(sm + L.sums) + warp * 2 * (g.K + g.R + 1);
     float *cf = sf + g.K;
+    const int p_of = lane / g.nq, q_of = lane % g.nq;
     build_next(sm, L, g);
 
     for (int64_t c = blockIdx.x; c < args.nchunks; c = next_chunk(args, c, next_slot)) {
@@ -424,13 +458,24 @@ __global__ void __launch_bounds__(kGBlock, lane_min_blocks<SPL, NT>()) generic_i
         unsigned n_eval = 0;
         // sample offsets in the chunk are 32-bit (a chunk never crosses a multiple of 2^32)
         const uint32_t cnt = static_cast<uint32_t>(v.cnt), xb = static_cast<uint32_t>(v.first);
+        int drawn = 0;  // SPL = 0: points in hand behind uf
+        uf = uf_all;
         for (uint32_t k0 = static_cast<uint32_t>(warp) * P; k0 < cnt; k0 += kGWarps * P) {
             // the screen of samples k0 .. k0 + P - 1 (group p of the warp screens k0 + p)
             float S_group;
             if constexpr (SPL > 0) {
                 S_group = scr.action(xb + k0 + (P > 1 ? lane / G : 0), word0, pre, ga.rk, ga.cf);
             } else {
-                warp_point<float>(v.first + k0, v.sid, ga.rk, g, [&](int j, uint32_t w) { return Coord<float>::map(w, bf[j].x, bf[j].y); }, uf);
+                if constexpr (!kBatch) {
+                    warp_point<float>(v.first + k0, v.sid, ga.rk, g, [&](int j, uint32_t w) { return Coord<float>::map(w, bf[j].x, bf[j].y); }, uf);
+                } else if (drawn == 0) {
+                    draw_points(v.first + k0, kGWarps, cnt - k0, v.sid, ga.rk, g, bf, p_of, q_of, uf_all);
+                    drawn = g.batch;
+                    uf = uf_all;
+                } else {
+                    uf += g.dpad;
+                }
+                drawn -= kBatch;
                 S_group = warp_action<float>(uf, next, g, ga.cf);
             }
 #pragma unroll
@@ -698,13 +743,23 @@ __global__ void __launch_bounds__(kGBlock) generic_hint(const GenArgs ga) {
     __syncthreads();
     const uint16_t *next = reinterpret_cast<const uint16_t *>(sm + L.next);
     const float2 *bf = reinterpret_cast<const float2 *>(sm + L.box_f);
-    float *uf = reinterpret_cast<float *>(sm + L.uf) + warp * g.dpad;
+    float *uf = reinterpret_cast<float *>(sm + L.uf) + warp * g.dpad * g.batch;
     const uint32_t sid = args.sub_id ? args.sub_id[s] : static_cast<uint32_t>(s);
     float mn = INFINITY;
-    for (uint64_t k = blockIdx.y * kGWarps + warp; k < n; k += gridDim.y * kGWarps) {
-        warp_point<float>(k, sid, ga.rk, g, [&](int j, uint32_t w) { return Coord<float>::map(w, bf[j].x, bf[j].y); }, uf);
-        mn = fminf(mn, warp_action<float>(uf, next, g, ga.cf));
-        __syncwarp();
+    const uint64_t step = gridDim.y * kGWarps;
+    if (g.batch == 1) {
+        for (uint64_t k = blockIdx.y * kGWarps + warp; k < n; k += step) {
+            warp_point<float>(k, sid, ga.rk, g, [&](int j, uint32_t w) { return Coord<float>::map(w, bf[j].x, bf[j].y); }, uf);
+            mn = fminf(mn, warp_action<float>(uf, next, g, ga.cf));
+            __syncwarp();
+        }
+    } else {
+        for (uint64_t k = blockIdx.y * kGWarps + warp; k < n; k += step * g.batch) {
+            draw_points(k, step, n - k, sid, ga.rk, g, bf, lane / g.nq, lane % g.nq, uf);
+            for (int p = 0; p < g.batch && k + p * step < n; ++p)
+                mn = fminf(mn, warp_action<float>(uf + p * g.dpad, next, g, ga.cf));
+            __syncwarp();
+        }
     }
     if (lane == 0) atomicMin(s_min, __float_as_int(mn));
     __syncthreads();
@@ -722,7 +777,7 @@ __global__ void __launch_bounds__(kGBlock) generic_eval(const EvalArgs a, const 
     const int64_t i = blockIdx.x * static_cast<int64_t>(kGWarps) + warp;
     if (i >= a.npts) return;  // warp-uniform
     const uint16_t *next = reinterpret_cast<const uint16_t *>(sm + L.next);
-    float *uf = reinterpret_cast<float *>(sm + L.uf) + warp * g.dpad;
+    float *uf = reinterpret_cast<float *>(sm + L.uf) + warp * g.dpad * g.batch;
     double *ud = reinterpret_cast<double *>(sm + L.ud) + warp * g.dpad;
     for (int j = lane; j < g.d; j += 32) {
         ud[j] = a.y[i * g.d + j];
@@ -815,6 +870,10 @@ cudaError_t mapped_occupancy(int nx, int nt, int *blocks_per_sm) {
 
 const ShapeKernels kGeneric = {0, 0, 1, {gen_integrand_launcher<true>, gen_integrand_launcher<false>},
                                {gen_occupancy<true>, gen_occupancy<false>}, gen_eval, nullptr, nullptr, nullptr, nullptr, 0};
+// up to 16 Philox blocks (d <= 64): the kernel that draws several points at once
+const ShapeKernels kGenericBatch = {0, 0, 1, {gen_integrand_launcher<true, 0, 1>, gen_integrand_launcher<false, 0, 1>},
+                                    {gen_occupancy<true, 0, 1>, gen_occupancy<false, 0, 1>}, gen_eval, nullptr, nullptr,
+                                    nullptr, nullptr, 0};
 
 // Shapes with Nx = G SPL and SPL NT in {4, 8, 16}: the register-resident
 // screen.  The shapes whose lanes would own one Philox block each (32x4, 64x2,
@@ -848,7 +907,7 @@ const ShapeKernels *generic_shape(int nx, int nt) {
     if (nx < 2 || nt < 1 || nx * nt > kMaxD) return nullptr;
     for (const ShapeKernels &k : kLanes)
         if (k.nx == nx && k.nt == nt) return &k;
-    return &kGeneric;
+    return nx * nt <= 64 ? &kGenericBatch : &kGeneric;
 }
 
 }  // namespace bfi
