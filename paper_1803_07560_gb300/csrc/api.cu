@@ -197,25 +197,35 @@ void plan_bind(bfi_plan &p, unsigned char *base, const PlanBytes &b) {
     p.d_partials = reinterpret_cast<double *>(base + b.part);
 }
 
+// Checks of a job that need no device.
+bfi_status plan_check(const bfi_lattice *lattice, int64_t nsub, const uint64_t *samples, bfi_precision precision,
+                      uint64_t *total, uint64_t *n_max) {
+    if (precision != BFI_FP64 && precision != BFI_FP32) return fail(BFI_E_INVALID, "unknown precision %d", precision);
+    if (!bfi::find_shape(lattice->nx, lattice->nt))
+        return fail(BFI_E_UNSUPPORTED, "lattice %dx%d has no compiled kernel in this library", lattice->nx,
+                    lattice->nt);
+    *total = 0;
+    *n_max = 1;
+    for (int64_t s = 0; s < nsub; ++s) {
+        if (samples[s] >= (1ull << 48))
+            return fail(BFI_E_INVALID, "samples[%lld] = %llu must be < 2^48", static_cast<long long>(s),
+                        static_cast<unsigned long long>(samples[s]));
+        *total += samples[s];
+        *n_max = std::max<uint64_t>(*n_max, samples[s]);
+    }
+    if (*total >= (1ull << 62)) return fail(BFI_E_INVALID, "total sample budget too large");
+    return BFI_OK;
+}
+
 // Checks the job and fills everything of the plan but its device memory, with
 // the box sampler; 'tables' gets the chunk table and the budgets.  The device
 // is current.
 bfi_status plan_describe(bfi_plan *p, const bfi_lattice *lattice, int64_t nsub, const uint64_t *samples,
                          bfi_precision precision, int device, std::vector<int64_t> &tables) {
-    if (precision != BFI_FP64 && precision != BFI_FP32) return fail(BFI_E_INVALID, "unknown precision %d", precision);
-    const bfi::ShapeKernels *shape = bfi::find_shape(lattice->nx, lattice->nt);
-    if (!shape)
-        return fail(BFI_E_UNSUPPORTED, "lattice %dx%d has no compiled kernel in this library", lattice->nx,
-                    lattice->nt);
     uint64_t total = 0, n_max = 1;
-    for (int64_t s = 0; s < nsub; ++s) {
-        if (samples[s] >= (1ull << 48))
-            return fail(BFI_E_INVALID, "samples[%lld] = %llu must be < 2^48", static_cast<long long>(s),
-                        static_cast<unsigned long long>(samples[s]));
-        total += samples[s];
-        n_max = std::max<uint64_t>(n_max, samples[s]);
-    }
-    if (total >= (1ull << 62)) return fail(BFI_E_INVALID, "total sample budget too large");
+    const bfi_status st = plan_check(lattice, nsub, samples, precision, &total, &n_max);
+    if (st != BFI_OK) return st;
+    const bfi::ShapeKernels *shape = bfi::find_shape(lattice->nx, lattice->nt);
     p->device = device;
     p->lat = to_params(lattice);
     p->precision = precision;
@@ -287,7 +297,8 @@ bfi_status bfi_plan_create(bfi_plan **out, const bfi_lattice *lattice, int64_t n
     if (st != BFI_OK) return st;
     if (nsub < 1) return fail(BFI_E_INVALID, "nsub must be >= 1 (got %lld)", static_cast<long long>(nsub));
     if (!samples) return fail(BFI_E_INVALID, "samples is NULL");
-    if (precision != BFI_FP64 && precision != BFI_FP32) return fail(BFI_E_INVALID, "unknown precision %d", precision);
+    uint64_t total = 0, n_max = 1;
+    if ((st = plan_check(lattice, nsub, samples, precision, &total, &n_max)) != BFI_OK) return st;
     DeviceGuard g(device);
     if (g.err != cudaSuccess) return fail(BFI_E_CUDA, "cannot select device %d: %s", device, cudaGetErrorString(g.err));
     bfi_plan *p = new (std::nothrow) bfi_plan();
