@@ -75,11 +75,16 @@ struct LogProduct {
 //     then has |dR| <= (2 eps + 8 u) T, T the sum of its terms' magnitudes with
 //     a for |v|; the bound used is E = 2^-17 T, 1.8 times that.
 //     S between inv sum max(0, |R| - E)^2 and inv sum (|R| + E)^2.
-//   * ln J, J = prod (1 + y^2) r^2, one logarithm per Philox block: 1e-3 and
-//     2^-15 of it cover the products' errors and lg2.approx's.
+//   * ln J = ln prod (1 + y^2) + 2 ln prod r, one logarithm for the first
+//     product (at most 2^D) and one per Philox block for the second: 1e-3 and
+//     2^-15 of it cover the products' errors and lg2.approx's.  (Products of
+//     (1 + y^2) r^2 pass 2^128 where the r of a block pass 2^62 together, in
+//     boxes of width 2^-8 next to 1 about once in 2^20 samples.)
 // The interval is a few thousandths wide for samples that matter, and it
-// grows with the terms that cancel in a residual; an overflow gives S_lo =
-// inf (true actions beyond 1e38) or NaN, which no comparison rejects.
+// grows with the terms that cancel in a residual.  Overflows: residuals give
+// S_lo = inf (true actions beyond 1e38) or NaN, which no comparison rejects,
+// and S_hi = inf or NaN; a product of r that is not finite bounds nothing,
+// [-inf, inf].
 // ---------------------------------------------------------------------------
 struct MapBox {
     float p0, m0, w;  // 1 + lo, 1 - hi, hi - lo
@@ -110,12 +115,12 @@ __device__ __forceinline__ void transform_screen(uint32_t x, const PhiloxPrefix 
     constexpr int D = NX * NT, NQ = (D + 3) / 4;
     const PhiloxFirst first = philox_first(x, pre[NQ].g);
     float v[D];
-    float ln_j = 0.f;
+    float ln_r = 0.f, one_y2 = 1.f;  // log2 prod r; prod (1 + y^2)
 #pragma unroll
     for (int q = 0; q < NQ; ++q) {
         const uint4 b = philox_from_prefix(first, pre[q], rk);
         const uint32_t w4[4] = {b.x, b.y, b.z, b.w};
-        float jac = 1.f;
+        float rs = 1.f;
 #pragma unroll
         for (int t = 0; t < 4; ++t) {
             const int j = 4 * q + t;
@@ -126,12 +131,13 @@ __device__ __forceinline__ void transform_screen(uint32_t x, const PhiloxPrefix 
                 const float p = fmaf(u, bx.w, bx.p0), m = fmaf(u1, bx.w, bx.m0);
                 const float r = rcp_approx(p * m), y = 0.5f * (p - m);
                 v[j] = y * r;
-                jac *= fmaf(y, y, 1.f) * (r * r);
+                one_y2 *= fmaf(y, y, 1.f);
+                rs *= r;
             }
         }
-        ln_j += __log2f(jac);
+        ln_r += __log2f(rs);
     }
-    ln_j *= 0.69314718f;
+    const float ln_j = 0.69314718f * fmaf(2.f, ln_r, __log2f(one_y2));
     const float a_adv = fabsf(c.c_adv), a_k1 = fabsf(c.k1), a_dif = fabsf(c.neg_c_dif);
     float low = 0.f, high = 0.f;
 #pragma unroll
@@ -165,6 +171,10 @@ __device__ __forceinline__ void transform_screen(uint32_t x, const PhiloxPrefix 
     }
     S_lo = fmaf(low, 1.f - 0x1p-15f, -fmaf(ln_j, 1.f + 0x1p-15f, 1e-3f));
     S_hi = fmaf(high, 1.f + 0x1p-15f, -fmaf(ln_j, 1.f - 0x1p-15f, -1e-3f));
+    if (!(ln_j < INFINITY)) {
+        S_lo = -INFINITY;
+        S_hi = INFINITY;
+    }
 }
 
 // Floats as integers in the same order (NaN aside), for atomicMin.
