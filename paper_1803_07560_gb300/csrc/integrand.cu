@@ -46,8 +46,9 @@ namespace bfi {
 // since a CTA's warps share the SM's FP64 pipe.
 constexpr int kMergeSpread = 152;
 constexpr int kMergeThreads = 512, kMergeWarps = kMergeThreads / 32;
-// a weightless subvolume, and one whose box has no volume (no finite log)
-constexpr int kNoWeight = INT_MIN, kNoVolume = INT_MIN + 1;
+// kexp of a weightless subvolume, and of one whose |ls| is beyond kFarLog or not finite (see finish_subvolume)
+constexpr int kNoWeight = INT_MIN, kFar = INT_MAX;
+constexpr double kFarLog = 0x1p29;
 
 __device__ __forceinline__ double warp_sum_f64(double v) {
 #pragma unroll
@@ -104,10 +105,13 @@ __device__ __forceinline__ double merge_list(int64_t count, int R, At at, Put pu
 
 // The slot of a subvolume (its sums are in slot[3 ...], unscaled products
 // Q_r = d P_r) and what the totals need of it:
-//   ls = log V - log n - m = kexp ln 2 + ln t, t in [1, 2) up to rounding, so
+//   ls = log V - log n - m = kexp ln 2 + ln t, t in [2^-1/2, 2^1/2], so
 //   that f_s / 2^kmax = t 2^(kexp - kmax) once the largest kexp is known;
 //   f_buf[s] = t, f_buf[nsub + s] = t^2 / (n - 1), and, in the place of the
-//   subvolume's first chunk record, kexp, V_Z, V_N(r) and Cov(r) without f.
+//   subvolume's first chunk record, kexp, V_Z, V_N(r), Cov(r) without f, and ls.
+// An ls that has no such kexp (a box without volume, or an action that leaves
+// |ls| >= kFarLog, as tiny D do) makes merge_slots take f_s = exp(ls - max ls)
+// of every subvolume itself.
 __device__ __forceinline__ void finish_subvolume(const MergeArgs &a, int64_t s, double m) {
     const int lane = threadIdx.x & 31, R = a.R, K = sum_count(R);
     double *slot = a.slots + s * (K + 3);
@@ -145,18 +149,18 @@ __device__ __forceinline__ void finish_subvolume(const MergeArgs &a, int64_t s, 
     }
     __syncwarp();
     const double sw = slot[3], sw2 = slot[4];
-    double tt = 0.0, gt = 0.0;
+    double tt = 0.0, gt = 0.0, ls = 0.0;
     int kexp = kNoWeight;
     if (n > 0.0 && sw > 0.0) {
-        const double ls = log_vol - log_n - m;
-        if (ls == -INFINITY) {
-            kexp = kNoVolume;
-            tt = 1.0;
-        } else {
-            // ln 2 in two parts, k times the upper one exact for |k| < 2^20
+        ls = log_vol - log_n - m;
+        if (fabs(ls) < kFarLog) {
+            // ln 2 in two parts, the upper one of 32 bits (Cody & Waite's reduction): ls - k upper is exact
             const double k = rint(ls * 1.4426950408889634);
             tt = exp(fma(-k, 1.9082149292705877e-10, fma(-k, 0.69314718036912382, ls)));
-            kexp = isfinite(ls) ? static_cast<int>(fmin(fmax(k, -1e9), 1e9)) : 0;  // not finite: tt is NaN
+            kexp = static_cast<int>(k);
+        } else {
+            kexp = kFar;
+            tt = 1.0;
         }
         if (n >= 2.0) gt = tt * tt / (n - 1.0);
     }
@@ -169,6 +173,7 @@ __device__ __forceinline__ void finish_subvolume(const MergeArgs &a, int64_t s, 
         if (room) {
             q[0] = static_cast<double>(kexp);
             q[1] = n * sw2 - sw * sw;
+            q[2 + 2 * R] = ls;
         }
     }
     for (int r = lane; r < R; r += 32) {
@@ -204,6 +209,17 @@ __device__ void merge_slots(const MergeArgs &a) {
     if (kmax != kNoWeight) atomicMax(&s_kmax, kmax);
     __syncthreads();
     kmax = s_kmax;
+    double lmax = -INFINITY;
+    if (kmax == kFar) {
+        for (int64_t s = tid; s < nsub; s += kMergeThreads)
+            if (!is_zero(__ldcg(a.f_buf + s))) lmax = fmax(lmax, __ldcg(record(s) + 2 + 2 * R));
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) lmax = fmax(lmax, __shfl_xor_sync(0xffffffffu, lmax, off));
+        if (lane == 0) sh[0][warp] = lmax;
+        __syncthreads();
+        for (int w = 0; w < kMergeWarps; ++w) lmax = fmax(lmax, sh[0][w]);
+        __syncthreads();
+    }
     double z = 0.0, vz = 0.0;
     unsigned long long n_tot = 0;
     int used = 0, bad = 0;
@@ -214,12 +230,13 @@ __device__ void merge_slots(const MergeArgs &a) {
         used += n > 0;
         if (!is_zero(f)) {
             const double *q = record(s);
-            const int k = static_cast<int>(__ldcg(q));
-            if (k == kNoVolume) {
-                f = g = kmax == kNoVolume ? NAN : 0.0;
+            if (kmax == kFar) {
+                f = exp(__ldcg(q + 2 + 2 * R) - lmax);
+                g = n < 2 ? 0.0 : f * f / (static_cast<double>(n) - 1.0);
             } else {
-                f *= pow2(k - kmax);
-                g *= pow2(2 * max(k - kmax, -1100));
+                const int k = static_cast<int>(__ldcg(q)) - kmax;
+                f *= pow2(k);
+                g *= pow2(2 * max(k, -1100));
             }
             z = fma(f, __ldcg(a.slots + s * SL + 3), z);
             if (n < 2) bad = 1;
@@ -273,6 +290,7 @@ __device__ void merge_slots(const MergeArgs &a) {
         const double Z = s_all[0];
         if (lane == 0)
             a.totals[0] = kmax == kNoWeight ? -INFINITY
+                          : kmax == kFar    ? lmax + log(Z)
                                             : fma(static_cast<double>(kmax), 0.69314718055994531, log(Z));
         else
             a.totals[1] = inf_err ? INFINITY : sqrt(s_all[1] > 0.0 ? s_all[1] : 0.0) / Z;
