@@ -1,6 +1,7 @@
 """The range map over boxes next to y = +-1, where v and the Jacobian grow
-without bound: slabs whose samples' FP32 Jacobian products overflow, records
-and shifts against the plain FP64 estimator and the shift rule."""
+without bound: slabs whose samples' FP32 Jacobian products overflow, and slabs
+whose samples' intervals are about as wide as a record's margin, records and
+shifts against the plain FP64 estimator and the shift rule."""
 import numpy as np
 import pytest
 
@@ -103,3 +104,34 @@ def test_path(bfi, nx, nt, k):
     lat, sid, one = bfi.lattice(nx, nt), np.zeros(1, dtype=np.uint32), np.ones((1, d))
     assert 0 < _run(bfi, lat, -one, one, n, 3, sid)[2] < 40_001 // 2
     assert _run(bfi, lat, one - 2.0 ** -k, one, n, 3, sid)[2] == 40_001
+
+
+@pytest.mark.parametrize("nx,nt,D,k,n", [
+    (2, 2, 4.0 ** 12, 12, 20_000), (2, 2, 1e6, 12, 1 << 21), (2, 2, 4.0 ** 16, 16, 1 << 15), (4, 2, 4.0 ** 18, 12, 70_001),
+    (2, 2, 4.0 ** 16, 16, 1 << 22)])
+def test_open_threads(bfi, nx, nt, D, k, n):
+    """Slabs where samples may or may not have moved their threads' shifts."""
+    d = nx * nt
+    _check(bfi, nx, nt, 0.1, D, 1.0, np.full((2, d), 1.0 - 2.0 ** -k), np.ones((2, d)), np.array([n, 700], dtype=np.uint64))
+
+
+def test_open_threads_time(bfi):
+    """Following the open threads costs no more than a few times an evaluation of every sample (which a box that
+    leaves [-1, 1] gets)."""
+    lat, n, dev = bfi.lattice(2, 2, D=4.0 ** 16), np.full(8, 1 << 15, dtype=np.uint64), torch.device("cuda:0")
+    plan = bfi.Plan(lat, n, bfi.FP64)
+    plan.set_sampler(bfi.SAMPLE_TRANSFORM)
+    hi = torch.ones((8, 4), dtype=torch.float64, device=dev)
+    ms = []
+    for lo in (hi - 2.0 ** -16, -1.5 * hi):
+        times = []
+        for _ in range(7):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            plan.execute(lo, hi, 9)
+            b.record()
+            torch.cuda.synchronize()
+            times.append(a.elapsed_time(b))
+        ms.append(min(times[2:]))
+    plan.close()
+    assert ms[0] < 3.0 * ms[1], ms
