@@ -66,26 +66,34 @@ struct LogProduct {
 // FP32 screen of the range map, with bounds.  For a box inside [-1, 1]^d it
 // returns S_lo and S_hi around the S_eff that the FP64 evaluation computes
 // (u = 2^-24 below; "relative" errors are to first order):
-//   * 1 + y = (1 + lo) + W u and 1 - y = (1 - hi) + W (1 - u) are sums of
-//     non-negative terms, u from the word and 1 - u from its complement, so
-//     both have a small relative error (5 u) however close y is to +-1;
-//     r = 1 / ((1 + y)(1 - y)), v = y r: |dv| <= eps a, a = |v| + 1, with
-//     eps = 32 u, which also covers the rounding of y in the evaluation.
+//   * p = 1 + y = (1 + lo) + W u and m = 1 - y = (1 - hi) + W (1 - u) are sums
+//     of non-negative terms, u from the word and 1 - u from its complement, so
+//     both have a relative error of 4 u, r = 1 / (p m) of 11 u, and v = y r an
+//     error of 17 u a, a = |v| + 1 >= r.
+//   * The evaluation rounds y, and with it 1 -+ y, by up to 2^-52 (its last
+//     bit, the rounding of W and of 1 + lo): v by 2^-51 r a, 8 u f a with
+//     f = max(1, 2^-30 r of the sample's largest r).  Together |dv| <= eps a,
+//     eps = 32 u f.
 //   * The residual R = v_next + v (c_adv (v_r - v_l) + k1) - c_dif (v_r + v_l)
 //     then has |dR| <= (2 eps + 8 u) T, T the sum of its terms' magnitudes with
-//     a for |v|; the bound used is E = 2^-17 T, 1.8 times that.
+//     a for |v|; the bound used is E = 2^-17 f T, 1.8 times that.
 //     S between inv sum max(0, |R| - E)^2 and inv sum (|R| + E)^2.
 //   * ln J = ln prod (1 + y^2) + 2 ln prod r, one logarithm for the first
-//     product (at most 2^D) and one per Philox block for the second: 1e-3 and
-//     2^-15 of it cover the products' errors and lg2.approx's.  (Products of
-//     (1 + y^2) r^2 pass 2^128 where the r of a block pass 2^62 together, in
-//     boxes of width 2^-8 next to 1 about once in 2^20 samples.)
+//     product (at most 2^D) and one per Philox block for the second: 1e-3 f and
+//     2^-15 of it cover the products' errors, y's rounding and lg2.approx's.
+//     (Products of (1 + y^2) r^2 pass 2^128 where the r of a block pass 2^62
+//     together, in boxes of width 2^-8 next to 1 about once in 2^20 samples.)
+//   * A sample with an r beyond kMapMaxR (y within 2^-41 of +-1, one coordinate
+//     in 2^41 over (-1, 1) and in 2^41 w over a slab of width w next to 1),
+//     where these are no longer small, or with a product of r that overflows,
+//     has no bound, [-inf, inf]: it is evaluated.
 // The interval is a few thousandths wide for samples that matter, and it
 // grows with the terms that cancel in a residual.  Overflows: residuals give
 // S_lo = inf (true actions beyond 1e38) or NaN, which no comparison rejects,
-// and S_hi = inf or NaN; a product of r that is not finite bounds nothing,
-// [-inf, inf].
+// and S_hi = inf or NaN.
 // ---------------------------------------------------------------------------
+constexpr float kMapMaxR = 0x1p40f;
+
 struct MapBox {
     float p0, m0, w;  // 1 + lo, 1 - hi, hi - lo
 };
@@ -115,7 +123,7 @@ __device__ __forceinline__ void transform_screen(uint32_t x, const PhiloxPrefix 
     constexpr int D = NX * NT, NQ = (D + 3) / 4;
     const PhiloxFirst first = philox_first(x, pre[NQ].g);
     float v[D];
-    float ln_r = 0.f, one_y2 = 1.f;  // log2 prod r; prod (1 + y^2)
+    float ln_r = 0.f, one_y2 = 1.f, r_max = 0.f;  // log2 prod r; prod (1 + y^2)
 #pragma unroll
     for (int q = 0; q < NQ; ++q) {
         const uint4 b = philox_from_prefix(first, pre[q], rk);
@@ -133,11 +141,13 @@ __device__ __forceinline__ void transform_screen(uint32_t x, const PhiloxPrefix 
                 v[j] = y * r;
                 one_y2 *= fmaf(y, y, 1.f);
                 rs *= r;
+                r_max = fmaxf(r_max, r);
             }
         }
         ln_r += __log2f(rs);
     }
     const float ln_j = 0.69314718f * fmaf(2.f, ln_r, __log2f(one_y2));
+    const float f = fmaxf(1.f, 0x1p-30f * r_max), eps = 0x1p-17f * f;
     const float a_adv = fabsf(c.c_adv), a_k1 = fabsf(c.k1), a_dif = fabsf(c.neg_c_dif);
     float low = 0.f, high = 0.f;
 #pragma unroll
@@ -151,7 +161,7 @@ __device__ __forceinline__ void transform_screen(uint32_t x, const PhiloxPrefix 
             const float side = fabsf(right) + fabsf(left) + 2.f;
             float T = fmaf(fabsf(here) + 1.f, fmaf(a_adv, side, a_k1), fabsf(next) + 1.f);
             T = fmaf(a_dif, side, T);
-            const float over = fmaf(0x1p-17f, T, fabsf(R)), under = fmaxf(fmaf(-0x1p-17f, T, fabsf(R)), 0.f);
+            const float over = fmaf(eps, T, fabsf(R)), under = fmaxf(fmaf(-eps, T, fabsf(R)), 0.f);
             low = fmaf(under, under, low);
             high = fmaf(over, over, high);
         }
@@ -162,16 +172,16 @@ __device__ __forceinline__ void transform_screen(uint32_t x, const PhiloxPrefix 
         float s_lo = 0.f, s_hi = 0.f;
 #pragma unroll
         for (int j = 0; j < D; ++j) {
-            const float a = fabsf(v[j]), e = fmaf(0x1p-18f, a, 0x1p-18f), under = fmaxf(a - e, 0.f), over = a + e;
+            const float a = fabsf(v[j]), e = 0.5f * fmaf(eps, a, eps), under = fmaxf(a - e, 0.f), over = a + e;
             s_lo = fmaf(under, under, s_lo);
             s_hi = fmaf(over, over, s_hi);
         }
         low = fmaf(c.half_mass2, s_lo, low);
         high = fmaf(c.half_mass2, s_hi, high);
     }
-    S_lo = fmaf(low, 1.f - 0x1p-15f, -fmaf(ln_j, 1.f + 0x1p-15f, 1e-3f));
-    S_hi = fmaf(high, 1.f + 0x1p-15f, -fmaf(ln_j, 1.f - 0x1p-15f, -1e-3f));
-    if (!(ln_j < INFINITY)) {
+    S_lo = fmaf(low, 1.f - 0x1p-15f, -fmaf(ln_j, 1.f + 0x1p-15f, 1e-3f * f));
+    S_hi = fmaf(high, 1.f + 0x1p-15f, -fmaf(ln_j, 1.f - 0x1p-15f, -1e-3f * f));
+    if (r_max > kMapMaxR || !(ln_j < INFINITY)) {
         S_lo = -INFINITY;
         S_hi = INFINITY;
     }
@@ -186,9 +196,10 @@ __device__ __forceinline__ float unorder_f32(int b) { return __int_as_float(b ^ 
 
 // Reference action of a subvolume: the smallest S_hi among its first
 // hint_samples(n_s) samples, or +inf where the screen is not to be used (its
-// premises fail, or the interval of that sample is wider than kMapResolved, the
-// margin that moves a shift, as in slabs close to +-1): every sample of the
-// subvolume is then evaluated.  Measured on GB300 at nu = 6 (2^20 to 2^24
+// premises fail, or more than one in 256 of these samples has no bound, or the
+// interval of that sample is wider than kMapResolved, the margin that moves a
+// shift, as in slabs close to +-1): every sample of the subvolume is then
+// evaluated.  Measured on GB300 at nu = 6 (2^20 to 2^24
 // samples, intervals of 0.1 to 8): 10x2 20.4 ms at a limit of 0.05 against
 // 0.80 ms at 1, 4 and 16; 32x2 4.95 ms at 0.05, 4.75 at 4, 0.81 at 16.  One
 // CTA per subvolume.
@@ -199,6 +210,7 @@ __global__ void __launch_bounds__(kBlock) hint_transform(const IntegrandArgs arg
                                                          const RoundKeys rk) {
     constexpr int D = NX * NT, NQ = (D + 3) / 4;
     __shared__ int s_min, s_low, s_bad;
+    __shared__ unsigned s_unbound;
     __shared__ MapBox s_map[D];
     __shared__ PhiloxPrefix s_pre[NQ + 1];
     const int64_t s = blockIdx.x;
@@ -206,6 +218,7 @@ __global__ void __launch_bounds__(kBlock) hint_transform(const IntegrandArgs arg
     if (tid == 0) {
         s_min = s_low = order_f32(INFINITY);
         s_bad = map_consts_screen(lc) ? 0 : 1;
+        s_unbound = 0u;
     }
     __syncthreads();
     const uint32_t sid = args.sub_id ? args.sub_id[s] : static_cast<uint32_t>(s);
@@ -223,14 +236,18 @@ __global__ void __launch_bounds__(kBlock) hint_transform(const IntegrandArgs arg
         float lo, hi;
         transform_screen<NX, NT>(k, s_pre, rk, s_map, lc, lo, hi);
         mn = fminf(mn, hi);
-        ln = fminf(ln, lo);
+        if (lo == -INFINITY)
+            atomicAdd(&s_unbound, 1u);
+        else
+            ln = fminf(ln, lo);
     }
     atomicMin(&s_min, order_f32(mn));
     atomicMin(&s_low, order_f32(ln));
     __syncthreads();
     if (tid == 0) {
         const float best = unorder_f32(s_min);
-        args.hint[s] = s_bad || !(best - unorder_f32(s_low) <= kMapResolved) ? INFINITY : best;
+        const bool bad = s_bad || 256u * s_unbound > n || !(best - unorder_f32(s_low) <= kMapResolved);
+        args.hint[s] = bad ? INFINITY : best;
     }
 }
 

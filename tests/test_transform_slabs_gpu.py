@@ -135,3 +135,20 @@ def test_open_threads_time(bfi):
         ms.append(min(times[2:]))
     plan.close()
     assert ms[0] < 3.0 * ms[1], ms
+
+
+@pytest.mark.parametrize("nx,nt,nonlinear,k,D,n", [
+    (2, 2, 1.0, 32, 2.0 ** 48, 1 << 18), (2, 2, 1.0, 34, 2.0 ** 52, 1 << 18), (10, 2, 0.0, 34, 2.0 ** 52, 1 << 16),
+    (2, 2, 1.0, 36, 2.0 ** 56, 5000), (2, 2, 1.0, 24, 2.0 ** 32, 1 << 18), (2, 2, 1.0, 12, 2.0 ** 8, 1 << 22)])
+def test_rounded_points(bfi, nx, nt, nonlinear, k, D, n):
+    """One coordinate within 2^-k of 1: samples so close to 1 that the rounding of y itself leaves the screen no bound
+    (1 / (1 - y^2) > 2^40) are evaluated, whatever their action."""
+    d = nx * nt
+    lo = -np.ones((1, d))
+    lo[0, 0] = 1.0 - 2.0 ** -k
+    facts, evaluated = _check(bfi, nx, nt, 0.1, D, nonlinear, lo, np.ones((1, d)), np.array([n], dtype=np.uint64))
+    y, S = facts[0]
+    r = (1.0 / ((1.0 - y) * (1.0 + y))).max(axis=1)
+    # the screen's 1 - y is not rounded as the evaluation's is: 2^-12 at 2^-41
+    needed = (S <= S.min() + 34.0 + np.log(n)) | (r > 2.0 ** 40 * (1.0 + 2.0 ** -11))
+    assert evaluated >= needed.sum(), (evaluated, needed.sum())
