@@ -638,7 +638,10 @@ bfi_status bfi_plan_get_timing(bfi_plan *plan, float *ms) {
 // 92 us; adaptive subdivision at 4x2 over 9 rounds 1.19 -> 0.80 ms.  Larger jobs'
 // arrays are copied directly: 300 subvolumes (104 KB) take 119 us so, 117 us
 // through the buffer, 1000 take 215 us either way, and a caller's own
-// page-locked arrays would be copied once more.
+// page-locked arrays would be copied once more.  Page-locking costs 100 us, ten
+// small calls' gain, so a context made for one call does without: creation and
+// first call take 249 us (324 with the buffer made at once), the second call
+// 233 (118), the later ones are the same.
 // ---------------------------------------------------------------------------
 constexpr size_t kStageBytes = size_t(64) << 10;
 
@@ -659,7 +662,8 @@ struct bfi_ctx {
     bfi_lattice lat{};
     unsigned char *buf = nullptr;
     size_t cap = 0;
-    unsigned char *stage = nullptr;  // page-locked, 2 kStageBytes: up, then down; null if it could not be had
+    unsigned char *stage = nullptr;  // page-locked, 2 kStageBytes: up, then down; made for the second small job
+    int64_t small_jobs = 0;
     int32_t sampler = BFI_SAMPLE_BOX;         // applied to every plan the context makes
     std::vector<double> map_mean, map_factor;
     std::vector<int64_t> tables;
@@ -720,10 +724,6 @@ bfi_status bfi_ctx_create(bfi_ctx **out, int device) {
     if (e != cudaSuccess) {
         delete c;
         return fail(BFI_E_CUDA, "cudaStreamCreate failed: %s", cudaGetErrorString(e));
-    }
-    if (cudaMallocHost(reinterpret_cast<void **>(&c->stage), 2 * kStageBytes) != cudaSuccess) {
-        cudaGetLastError();
-        c->stage = nullptr;
     }
     *out = c;
     return BFI_OK;
@@ -825,6 +825,12 @@ bfi_status bfi_integrate(bfi_ctx *ctx, const bfi_lattice *lattice, int64_t nsub,
                  n_slots = at.totals - at.slots, n_totals = sizeof(double) * bfi_totals_len(lattice->nx);
     const size_t up = sub_id ? at.up_end : at.sid, from = replan ? 0 : at.lo;
     const size_t down = slots ? n_slots + n_totals : n_totals;
+    // the second small job makes the buffer, and does without it for good if it cannot be had
+    if (up <= kStageBytes && ++ctx->small_jobs == 2 &&
+        cudaMallocHost(reinterpret_cast<void **>(&ctx->stage), 2 * kStageBytes) != cudaSuccess) {
+        cudaGetLastError();
+        ctx->stage = nullptr;
+    }
     const bool stage_up = ctx->stage && up <= kStageBytes, stage_down = ctx->stage && down <= kStageBytes;
     unsigned char *h_up = ctx->stage, *h_down = ctx->stage + kStageBytes;
     auto enqueue = [&]() -> bfi_status {
