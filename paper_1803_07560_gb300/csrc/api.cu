@@ -628,10 +628,13 @@ bfi_status bfi_plan_get_timing(bfi_plan *plan, float *ms) {
 }  // extern "C"
 
 // ---------------------------------------------------------------------------
-// Context: one device, one stream, a cached plan and one device buffer that
-// only grows, so that a caller whose jobs change from call to call (a round of
-// adaptive subdivision, a line of the line protocol) allocates nothing after
-// the largest.  A small job's chunk table and inputs go to the device in one
+// Context: one device, one stream, a cached plan and one device buffer kept
+// between calls, so that a caller whose jobs change from call to call (a round
+// of adaptive subdivision, a line of the line protocol) allocates no buffer
+// after the largest.  It is grown to twice its size, by kSlackBytes over the
+// job's need at most, and given back where a new job needs less than a quarter
+// of it and it holds more than kKeepBytes.  (A re-plan with the Gaussian sampler
+// still makes its factor's device memory anew.)  A small job's chunk table and inputs go to the device in one
 // copy through page-locked memory, and its records and totals come back in
 // one; a copy from or to pageable memory waits in the driver.  Measured on
 // GB300 at 10x2: 3 subvolumes (1 KB up) 89 -> 78 us a call, 100 (35 KB) 100 ->
@@ -644,6 +647,7 @@ bfi_status bfi_plan_get_timing(bfi_plan *plan, float *ms) {
 // 233 (118), the later ones are the same.
 // ---------------------------------------------------------------------------
 constexpr size_t kStageBytes = size_t(64) << 10;
+constexpr size_t kSlackBytes = size_t(16) << 20, kKeepBytes = size_t(64) << 20;
 
 // Byte offsets in the context's device buffer: what goes up (chunk table and
 // budgets, lo, hi, sub_id) and what comes down (slots, totals) lie together.
@@ -785,9 +789,10 @@ bfi_status bfi_integrate(bfi_ctx *ctx, const bfi_lattice *lattice, int64_t nsub,
         ctx->planned = false;
         if ((st = plan_describe(plan, lattice, nsub, samples, precision, ctx->device, ctx->tables)) != BFI_OK) return st;
         ctx->at = ctx_layout(*plan, *lattice);
-        if (ctx->at.total > ctx->cap) {
-            // twice the last size at least, so that growing jobs do not allocate on every call
-            const size_t want = std::max(ctx->at.total, std::min(2 * ctx->cap, ctx->at.total + (size_t(256) << 20)));
+        if (ctx->at.total > ctx->cap || (ctx->cap > kKeepBytes && ctx->at.total < ctx->cap / 4)) {
+            const size_t want = ctx->at.total < ctx->cap
+                                    ? ctx->at.total
+                                    : std::max(ctx->at.total, std::min(2 * ctx->cap, ctx->at.total + kSlackBytes));
             cudaFree(ctx->buf);
             ctx->buf = nullptr;
             ctx->cap = 0;

@@ -47,3 +47,28 @@ def test_kept_plan(bfi):
             assert np.array_equal(a_t, b_t, equal_nan=True), (n, i)
             assert not kw["want_slots"] or np.array_equal(a_s, b_s, equal_nan=True), (n, i)
         ctx.close()
+
+
+def test_device_memory(bfi):
+    """A context's buffer follows its jobs: little over a large job's need after a smaller one, and given back by a
+    small job."""
+    lat, small = bfi.lattice(10, 2), np.array([300], dtype=np.uint64)
+    one = np.ones((1, 20))
+
+    def free():
+        torch.cuda.synchronize()
+        return torch.cuda.mem_get_info(0)[0]
+
+    def large(ctx, n):
+        ctx.integrate(lat, np.repeat(-one, n, axis=0), np.repeat(one, n, axis=0), np.ones(n, dtype=np.uint64), 1)
+        return n * (2 * 8 * 20 + 8 * 23 + 8 * 22 + 44)  # boxes, slots, chunk records, tables and factors
+
+    ctx = bfi.Context(0)
+    ctx.integrate(lat, -one, one, small, 1)
+    before = free()
+    large(ctx, 200_000)
+    need = large(ctx, 210_000)
+    assert before - free() < need + (40 << 20), (before - free(), need)
+    ctx.integrate(lat, -one, one, small, 1)
+    assert abs(before - free()) <= 4 << 20, before - free()
+    ctx.close()
