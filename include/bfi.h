@@ -68,15 +68,19 @@
  *  - Negligible weights: a sample whose action exceeds the subvolume's
  *    smallest action by more than W = c + ln(n_max) (n_max the largest
  *    budget of the plan; c = 34 in BFI_FP64, 20 in BFI_FP32) has weight below
- *    e^-W of the largest, and all such samples together move any sum by less
- *    than e^-c relative.  They are counted in n_s but left out of the sums.
+ *    e^-W of the largest, and all such samples together move sum w by less
+ *    than e^-c relative, and a sum with P_r by less than e^-c max|P| / C(0)
+ *    of its r = 0 member, max|P| over the samples left out: at most vmax^2
+ *    for boxes of |v| <= vmax; the range map (see Samplers) sets no limit to
+ *    v, nor this to its P.  They are counted in n_s but left out of the sums.
  *    Both modes decide this from an FP32 action of a float point with a
  *    margin of 1 + 0.1% of S, far above its difference from the action the
- *    evaluation computes.
- *    The reference action starts at the smallest FP32 action among each
- *    subvolume's first n_s/32 samples (256 to 4096) and follows the smallest evaluated
- *    action, shared at fixed points of the sample loop, so the outcome is
- *    reproducible.
+ *    evaluation computes; the range map from FP32 bounds on the action that
+ *    the evaluation computes, sample by sample.
+ *    The reference action starts at the smallest FP32 action (range map: upper
+ *    bound) among each subvolume's first n_s/32 samples (256 to 4096) and
+ *    follows the smallest evaluated action, shared at fixed points of the
+ *    sample loop, so the outcome is reproducible.
  *  - Errors: every call returns a bfi_status; bfi_last_error() gives a
  *    message for the calling thread.  No call aborts the process.
  *

@@ -217,14 +217,12 @@ bfi_status plan_check(const bfi_lattice *lattice, int64_t nsub, const uint64_t *
     return BFI_OK;
 }
 
-// Checks the job and fills everything of the plan but its device memory, with
-// the box sampler; 'tables' gets the chunk table and the budgets.  The device
-// is current.
+// Fills everything of a checked job's plan but its device memory, with the box
+// sampler; 'tables' gets the chunk table and the budgets.  The device is
+// current; total and n_max are plan_check's.
 bfi_status plan_describe(bfi_plan *p, const bfi_lattice *lattice, int64_t nsub, const uint64_t *samples,
-                         bfi_precision precision, int device, std::vector<int64_t> &tables) {
-    uint64_t total = 0, n_max = 1;
-    const bfi_status st = plan_check(lattice, nsub, samples, precision, &total, &n_max);
-    if (st != BFI_OK) return st;
+                         bfi_precision precision, int device, uint64_t total, uint64_t n_max,
+                         std::vector<int64_t> &tables) {
     const bfi::ShapeKernels *shape = bfi::find_shape(lattice->nx, lattice->nt);
     p->device = device;
     p->lat = to_params(lattice);
@@ -304,7 +302,7 @@ bfi_status bfi_plan_create(bfi_plan **out, const bfi_lattice *lattice, int64_t n
     bfi_plan *p = new (std::nothrow) bfi_plan();
     if (!p) return fail(BFI_E_NOMEM, "host allocation failed");
     std::vector<int64_t> tables;
-    if ((st = plan_describe(p, lattice, nsub, samples, precision, device, tables)) != BFI_OK) {
+    if ((st = plan_describe(p, lattice, nsub, samples, precision, device, total, n_max, tables)) != BFI_OK) {
         delete p;
         return st;
     }
@@ -602,7 +600,7 @@ bfi_status bfi_plan_get_work(bfi_plan *plan, bfi_work *work) {
     const uint64_t total = static_cast<uint64_t>(plan->total);
     work->samples = total;
     work->evaluated = c[0];
-    if (plan->sampler != BFI_SAMPLE_BOX) {  // every sample evaluated, no screen
+    if (plan->sampler != BFI_SAMPLE_BOX) {  // the range map's own screen counts only what it lets through
         work->stage1 = work->full_screen = work->survivors = 0;
     } else {
         work->stage1 = c[2];
@@ -637,8 +635,8 @@ bfi_status bfi_plan_get_timing(bfi_plan *plan, float *ms) {
 // still makes its factor's device memory anew.)  A small job's chunk table and inputs go to the device in one
 // copy through page-locked memory, and its records and totals come back in
 // one; a copy from or to pageable memory waits in the driver.  Measured on
-// GB300 at 10x2: 3 subvolumes (1 KB up) 89 -> 78 us a call, 100 (35 KB) 100 ->
-// 92 us; adaptive subdivision at 4x2 over 9 rounds 1.19 -> 0.80 ms.  Larger jobs'
+// GB300 at 10x2: 3 subvolumes (1 KB up) 11 us less a call (84 to 89 us now, by
+// box and budgets), 100 (35 KB) 100 -> 92 us; adaptive subdivision at 4x2 over 9 rounds 1.19 -> 0.80 ms.  Larger jobs'
 // arrays are copied directly: 300 subvolumes (104 KB) take 119 us so, 117 us
 // through the buffer, 1000 take 215 us either way, and a caller's own
 // page-locked arrays would be copied once more.  Page-locking costs 100 us, ten
@@ -787,7 +785,10 @@ bfi_status bfi_integrate(bfi_ctx *ctx, const bfi_lattice *lattice, int64_t nsub,
     cudaStream_t s = ctx->stream;
     if (replan) {
         ctx->planned = false;
-        if ((st = plan_describe(plan, lattice, nsub, samples, precision, ctx->device, ctx->tables)) != BFI_OK) return st;
+        uint64_t total = 0, n_max = 1;
+        if ((st = plan_check(lattice, nsub, samples, precision, &total, &n_max)) != BFI_OK ||
+            (st = plan_describe(plan, lattice, nsub, samples, precision, ctx->device, total, n_max, ctx->tables)) != BFI_OK)
+            return st;
         ctx->at = ctx_layout(*plan, *lattice);
         if (ctx->at.total > ctx->cap || (ctx->cap > kKeepBytes && ctx->at.total < ctx->cap / 4)) {
             const size_t want = ctx->at.total < ctx->cap

@@ -128,7 +128,7 @@ template <int D>
 __device__ __forceinline__ void sample_words_pre(uint32_t x, const PhiloxPrefix *pre, const RoundKeys &rk,
                                                  uint32_t (&w)[D]) {
     constexpr int NQ = (D + 3) / 4;
-            const PhiloxFirst first = philox_first(x, pre[NQ].g);
+    const PhiloxFirst first = philox_first(x, pre[NQ].g);
 #pragma unroll
     for (int q = 0; q < NQ; ++q) {
         const uint4 b = philox_from_prefix(first, pre[q], rk);
@@ -143,7 +143,7 @@ template <int D>
 __device__ __forceinline__ void make_point_pre(uint32_t x, const PhiloxPrefix *pre, const RoundKeys &rk,
                                                const float2 *box, float (&u)[D]) {
     constexpr int NQ = (D + 3) / 4;
-        const PhiloxFirst first = philox_first(x, pre[NQ].g);
+    const PhiloxFirst first = philox_first(x, pre[NQ].g);
 #pragma unroll
     for (int q = 0; q < NQ; ++q) {
         const uint4 b = philox_from_prefix(first, pre[q], rk);
