@@ -11,6 +11,7 @@
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
+#include <cstdlib>
 #include <cstring>
 #include <string>
 #include <vector>
@@ -640,9 +641,9 @@ bfi_status bfi_plan_get_timing(bfi_plan *plan, float *ms) {
 // arrays are copied directly: 300 subvolumes (104 KB) take 119 us so, 117 us
 // through the buffer, 1000 take 215 us either way, and a caller's own
 // page-locked arrays would be copied once more.  Page-locking costs 100 us, ten
-// small calls' gain, so a context made for one call does without: creation and
-// first call take 249 us (324 with the buffer made at once), the second call
-// 233 (118), the later ones are the same.
+// small calls' gain, so a context made for one call goes through plain memory:
+// creation and first call take 230 us (325 with the buffer locked at once), the
+// second call 230 (117), later ones the same.
 // ---------------------------------------------------------------------------
 constexpr size_t kStageBytes = size_t(64) << 10;
 constexpr size_t kSlackBytes = size_t(16) << 20, kKeepBytes = size_t(64) << 20;
@@ -664,7 +665,8 @@ struct bfi_ctx {
     bfi_lattice lat{};
     unsigned char *buf = nullptr;
     size_t cap = 0;
-    unsigned char *stage = nullptr;  // page-locked, 2 kStageBytes: up, then down; made for the second small job
+    unsigned char *stage = nullptr;  // 2 kStageBytes: up, then down; page-locked from the second small job on
+    bool stage_locked = false;
     int64_t small_jobs = 0;
     int32_t sampler = BFI_SAMPLE_BOX;         // applied to every plan the context makes
     std::vector<double> map_mean, map_factor;
@@ -727,6 +729,7 @@ bfi_status bfi_ctx_create(bfi_ctx **out, int device) {
         delete c;
         return fail(BFI_E_CUDA, "cudaStreamCreate failed: %s", cudaGetErrorString(e));
     }
+    c->stage = static_cast<unsigned char *>(std::malloc(2 * kStageBytes));  // without it the arrays are copied directly
     *out = c;
     return BFI_OK;
 }
@@ -738,7 +741,8 @@ bfi_status bfi_ctx_destroy(bfi_ctx *ctx) {
         cudaStreamSynchronize(ctx->stream);
         cudaFree(ctx->buf);
         cudaFree(ctx->plan.d_map);
-        cudaFreeHost(ctx->stage);
+        if (ctx->stage_locked) cudaFreeHost(ctx->stage);
+        else std::free(ctx->stage);
         cudaStreamDestroy(ctx->stream);
     }
     delete ctx;
@@ -831,11 +835,15 @@ bfi_status bfi_integrate(bfi_ctx *ctx, const bfi_lattice *lattice, int64_t nsub,
                  n_slots = at.totals - at.slots, n_totals = sizeof(double) * bfi_totals_len(lattice->nx);
     const size_t up = sub_id ? at.up_end : at.sid, from = replan ? 0 : at.lo;
     const size_t down = slots ? n_slots + n_totals : n_totals;
-    // the second small job makes the buffer, and does without it for good if it cannot be had
-    if (up <= kStageBytes && ++ctx->small_jobs == 2 &&
-        cudaMallocHost(reinterpret_cast<void **>(&ctx->stage), 2 * kStageBytes) != cudaSuccess) {
-        cudaGetLastError();
-        ctx->stage = nullptr;
+    if (up <= kStageBytes && ++ctx->small_jobs == 2) {
+        void *locked = nullptr;
+        if (cudaMallocHost(&locked, 2 * kStageBytes) == cudaSuccess) {
+            std::free(ctx->stage);
+            ctx->stage = static_cast<unsigned char *>(locked);
+            ctx->stage_locked = true;
+        } else {
+            cudaGetLastError();  // the plain buffer stays
+        }
     }
     const bool stage_up = ctx->stage && up <= kStageBytes, stage_down = ctx->stage && down <= kStageBytes;
     unsigned char *h_up = ctx->stage, *h_down = ctx->stage + kStageBytes;
