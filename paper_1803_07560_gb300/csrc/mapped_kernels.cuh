@@ -622,7 +622,7 @@ __device__ __forceinline__ long long bound_key(double b) {
 // compiled for one CTA per SM with all the registers a thread may have.  At
 // 10x2 about 860 FP64 instructions a sample: 360 for the ten pairs, 210 for
 // F z, 120 for the action, 111 for the products, the rest for the weight and
-// the sums (883 counted, the pipe 91% busy; 1300 before the tables, the sums
+// the sums (869 counted, the pipe 91% busy; 1300 before the tables, the sums
 // by FMA and the box test off the pipe).  Measured on GB300, 2^22 samples at
 // 10x2: 9.94 -> 6.72 ms.
 // ---------------------------------------------------------------------------
