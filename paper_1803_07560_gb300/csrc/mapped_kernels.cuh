@@ -289,7 +289,9 @@ __global__ void __launch_bounds__(kBlock) hint_transform(const IntegrandArgs arg
 // scheduler, ~590 of them an evaluation, against ~1000 instructions of the
 // screen per row of 32 samples; two CTAs per SM let one's evaluations run
 // under the other's screen (lattices over 32 sites hold the FP64 field of an
-// evaluation in over 128 registers: one CTA).
+// evaluation in over 128 registers: one CTA; up to 4 sites three fit with 80,
+// and an open thread's shift lies in shared memory to keep it so: 2x2, 3000 x
+// 60 samples take 200 us, 235 at two CTAs).
 //
 // Measured on GB300 (whole pass, against the kernel that evaluated every
 // sample; nu = 1, [-1, 1]^d bisected): 10x2, 256 x 2^16 samples 19.55 ->
@@ -346,18 +348,17 @@ __global__ void __launch_bounds__(BLOCK, NX *NT <= 32 ? 2 : 1)
         const uint32_t cnt = static_cast<uint32_t>(v.cnt), xb = static_cast<uint32_t>(v.first);
         const uint32_t nrows = (cnt + BLOCK - 1) / BLOCK;
         bool ask = false;                           // this thread decides and its k_m has not been evaluated
-        bool walk = false;                          // this thread decides and is open: its shift is followed from
-        uint32_t from = 0u;                         // this sample on
-        double m_walk = INFINITY;
+        bool walk = false;                          // this thread decides and is open: its shift is followed, in
+                                                    // s_S, from sample s_km on (or from its first)
         // rows 0 .. nrows - 1; then the samples left in the queues; then the k_m that decide but were outside the
         // window; then the open threads' rows again, warp by warp
         for (uint32_t row = 0;;) {
             const bool again = row > nrows + 1;
             const uint32_t k = (again ? row - nrows - 2 : row) * BLOCK + tid;
-            const bool follows = again && walk && k >= from && k < cnt;
+            const bool follows = again && walk && k < cnt && (s_km[tid] == kNone || k >= s_km[tid]);
             uint32_t k_eval = 0u;
             float lo = -INFINITY, hi = INFINITY;
-            if (row < nrows ? k < cnt && !direct : follows && m_walk < INFINITY)
+            if (row < nrows ? k < cnt && !direct : follows && s_S[tid] < INFINITY)
                 transform_screen<NX, NT>(xb + k, s_pre, rk, s_map, lcf, lo, hi);
             bool evaluate = false;
             if (row < nrows) {
@@ -406,7 +407,7 @@ __global__ void __launch_bounds__(BLOCK, NX *NT <= 32 ? 2 : 1)
                 evaluate = ask;
                 if (ask) k_eval = s_km[tid];
             } else {
-                const float m = __double2float_ru(m_walk);
+                const float m = __double2float_ru(s_S[tid]);
                 evaluate = follows && !(lo >= m - kRescaleMargin + 0x1p-20f * fabsf(m));
                 k_eval = k;
             }
@@ -446,10 +447,8 @@ __global__ void __launch_bounds__(BLOCK, NX *NT <= 32 ? 2 : 1)
                     }
                     accumulate<K, R, BLOCK>(acc, exp(m_acc - S), Q);
                     ++n_eval;
-                } else if (!again) {
+                } else if (!again || S < s_S[tid] - kRescaleMargin) {
                     s_S[tid] = S;
-                } else if (S < m_walk - kRescaleMargin) {
-                    m_walk = S;
                 }
             }
             if (row < nrows) {
@@ -476,7 +475,7 @@ __global__ void __launch_bounds__(BLOCK, NX *NT <= 32 ? 2 : 1)
                 if (decides && known) atomicMin(&s_shift, order_f64(s_S[tid]));
                 ask = decides && !open && !known;
                 walk = decides && open;
-                from = s_km[tid] == kNone ? tid : s_km[tid];
+                if (walk) s_S[tid] = INFINITY;
                 if (__syncthreads_or(ask)) {
                     row = nrows + 1;
                     continue;
@@ -485,9 +484,10 @@ __global__ void __launch_bounds__(BLOCK, NX *NT <= 32 ? 2 : 1)
                 if (ask) atomicMin(&s_shift, order_f64(s_S[tid]));
             }
             // the walk: no barrier until every warp has left the loop
-            row = again ? row + 1 : nrows + 2 + __reduce_min_sync(0xffffffffu, walk ? from / BLOCK : nrows);
+            const uint32_t from = s_km[tid] == kNone ? 0u : s_km[tid] / BLOCK;
+            row = again ? row + 1 : nrows + 2 + __reduce_min_sync(0xffffffffu, walk ? from : nrows);
             if (row < 2 * nrows + 2) continue;
-            if (walk && m_walk < INFINITY) atomicMin(&s_shift, order_f64(m_walk));
+            if (walk) atomicMin(&s_shift, order_f64(s_S[tid]));  // +inf moves nothing
             break;
         }
         add_evaluated(args.stats, n_eval, &sh.evaluated);

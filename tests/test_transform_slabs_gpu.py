@@ -152,3 +152,12 @@ def test_rounded_points(bfi, nx, nt, nonlinear, k, D, n):
     # the screen's 1 - y is not rounded as the evaluation's is: 2^-12 at 2^-41
     needed = (S <= S.min() + 34.0 + np.log(n)) | (r > 2.0 ** 40 * (1.0 + 2.0 ** -11))
     assert evaluated >= needed.sum(), (evaluated, needed.sum())
+
+
+@pytest.mark.parametrize("nx,nt", [(2, 1), (3, 1), (4, 1), (2, 2)])
+def test_residency(bfi, nx, nt):
+    """The smallest lattices run three CTAs an SM (80 registers), which jobs of short chunks need."""
+    plan = bfi.Plan(bfi.lattice(nx, nt), np.array([300], dtype=np.uint64), bfi.FP64)
+    plan.set_sampler(bfi.SAMPLE_TRANSFORM)
+    assert plan.info().ctas_per_sm_max >= 3
+    plan.close()
