@@ -199,10 +199,15 @@ __device__ __forceinline__ float unorder_f32(int b) { return __int_as_float(b ^ 
 // premises fail, or more than one in 256 of these samples has no bound, or the
 // interval of that sample is wider than kMapResolved, the margin that moves a
 // shift, as in slabs close to +-1): every sample of the subvolume is then
-// evaluated.  Measured on GB300 at nu = 6 (2^20 to 2^24
-// samples, intervals of 0.1 to 8): 10x2 20.4 ms at a limit of 0.05 against
-// 0.80 ms at 1, 4 and 16; 32x2 4.95 ms at 0.05, 4.75 at 4, 0.81 at 16.  One
-// CTA per subvolume.
+// evaluated.  So it is where the screen gains nothing: where more than 15 in 16
+// of these samples lie within the window of the reference, or more than half
+// while the interval is wider than 8, which leaves most threads open.
+// Measured on GB300 at nu = 6 (2^20 to 2^24 samples, intervals of 0.1 to 8):
+// 10x2 20.4 ms at a limit of 0.05 against 0.80 ms at 1, 4 and 16; 32x2 4.95 ms
+// at 0.05, 4.75 at 4, 0.81 at 16.  At 2x2, 300 x 2000 samples screened and
+// evaluated throughout: [-1, 1]^4 with D = 4^8 309 and 269 us; [1 - 2^-20, 1]^4
+// with D = 4^25, all within the window, 390 and 266; at widths of 4 to 8 and
+// three in four samples 279 and 283.  One CTA per subvolume.
 constexpr float kMapResolved = 16.f;
 
 template <int NX, int NT>
@@ -210,7 +215,8 @@ __global__ void __launch_bounds__(kBlock) hint_transform(const IntegrandArgs arg
                                                          const RoundKeys rk) {
     constexpr int D = NX * NT, NQ = (D + 3) / 4;
     __shared__ int s_min, s_low, s_bad;
-    __shared__ unsigned s_unbound;
+    __shared__ unsigned s_unbound, s_near;
+    __shared__ float s_S[4096];  // S_lo of the samples
     __shared__ MapBox s_map[D];
     __shared__ PhiloxPrefix s_pre[NQ + 1];
     const int64_t s = blockIdx.x;
@@ -218,7 +224,7 @@ __global__ void __launch_bounds__(kBlock) hint_transform(const IntegrandArgs arg
     if (tid == 0) {
         s_min = s_low = order_f32(INFINITY);
         s_bad = map_consts_screen(lc) ? 0 : 1;
-        s_unbound = 0u;
+        s_unbound = s_near = 0u;
     }
     __syncthreads();
     const uint32_t sid = args.sub_id ? args.sub_id[s] : static_cast<uint32_t>(s);
@@ -235,6 +241,7 @@ __global__ void __launch_bounds__(kBlock) hint_transform(const IntegrandArgs arg
     for (uint32_t k = tid; k < n; k += kBlock) {
         float lo, hi;
         transform_screen<NX, NT>(k, s_pre, rk, s_map, lc, lo, hi);
+        s_S[k] = lo;
         mn = fminf(mn, hi);
         if (lo == -INFINITY)
             atomicAdd(&s_unbound, 1u);
@@ -244,9 +251,14 @@ __global__ void __launch_bounds__(kBlock) hint_transform(const IntegrandArgs arg
     atomicMin(&s_min, order_f32(mn));
     atomicMin(&s_low, order_f32(ln));
     __syncthreads();
+    const float best = unorder_f32(s_min), width = best - unorder_f32(s_low);
+    unsigned near = 0u;
+    for (uint32_t k = tid; k < n; k += kBlock) near += s_S[k] > __fadd_ru(best, args.skip_window) ? 0u : 1u;
+    atomicAdd(&s_near, near);
+    __syncthreads();
     if (tid == 0) {
-        const float best = unorder_f32(s_min);
-        const bool bad = s_bad || 256u * s_unbound > n || !(best - unorder_f32(s_low) <= kMapResolved);
+        const bool bad = s_bad || 256u * s_unbound > n || !(width <= kMapResolved) || 16u * s_near > 15u * n ||
+                         (width > 8.f && 2u * s_near > n);
         args.hint[s] = bad ? INFINITY : best;
     }
 }

@@ -107,7 +107,7 @@ def test_path(bfi, nx, nt, k):
 
 
 @pytest.mark.parametrize("nx,nt,D,k,n", [
-    (2, 2, 4.0 ** 12, 12, 20_000), (2, 2, 1e6, 12, 1 << 21), (2, 2, 4.0 ** 16, 16, 1 << 15), (4, 2, 4.0 ** 18, 12, 70_001),
+    (2, 2, 4.0 ** 12, 12, 20_000), (2, 2, 1e6, 12, 1 << 21), (2, 2, 1e6, 13, 70_001), (2, 2, 1e7, 14, 70_001), (2, 2, 4.0 ** 16, 16, 1 << 15), (4, 2, 4.0 ** 18, 12, 70_001),
     (2, 2, 4.0 ** 16, 16, 1 << 22)])
 def test_open_threads(bfi, nx, nt, D, k, n):
     """Slabs where samples may or may not have moved their threads' shifts."""
@@ -161,3 +161,13 @@ def test_residency(bfi, nx, nt):
     plan.set_sampler(bfi.SAMPLE_TRANSFORM)
     assert plan.info().ctas_per_sm_max >= 3
     plan.close()
+
+
+@pytest.mark.parametrize("k,D,screened", [(0, 1.0, True), (0, 4.0 ** 8, False), (12, 1e6, True), (16, 4.0 ** 16, False),
+                                          (20, 4.0 ** 30, False)])
+def test_where_the_screen_gains(bfi, k, D, screened):
+    """Every sample is evaluated where nearly all lie within the window, or many do and their intervals are wide."""
+    n, one = np.array([300_000], dtype=np.uint64), np.ones((1, 4))
+    lo = -one if k == 0 else one - 2.0 ** -k
+    evaluated = _run(bfi, bfi.lattice(2, 2, D=D), lo, one, n, 3, np.zeros(1, dtype=np.uint32))[2]
+    assert (evaluated < 300_000) == screened, evaluated
