@@ -544,8 +544,8 @@ bfi_status bfi_request_release(bfi_request *request);
  * integration request after another.  A context is used by one thread at a
  * time; a concurrent call returns BFI_E_BUSY.
  * Between calls it holds one device buffer of what its largest job needed, at
- * most 16 MiB more, and from its second small job on 128 KiB of page-locked
- * host memory.  A job that needs less than a quarter of a buffer of over
+ * most 16 MiB more, and from its second job whose inputs or results take up to
+ * 64 KiB on 128 KiB of page-locked host memory.  A job that needs less than a quarter of a buffer of over
  * 64 MiB gives the buffer back for one of its own size; bfi_ctx_destroy frees
  * all.
  * Errors: BFI_E_INVALID, BFI_E_NOMEM, BFI_E_CUDA. */

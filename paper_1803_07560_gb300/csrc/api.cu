@@ -665,7 +665,7 @@ struct bfi_ctx {
     bfi_lattice lat{};
     unsigned char *buf = nullptr;
     size_t cap = 0;
-    unsigned char *stage = nullptr;  // 2 kStageBytes: up, then down; page-locked from the second small job on
+    unsigned char *stage = nullptr;  // 2 kStageBytes: up, then down; page-locked from the second job that uses it on
     bool stage_locked = false;
     int64_t small_jobs = 0;
     int32_t sampler = BFI_SAMPLE_BOX;         // applied to every plan the context makes
@@ -835,7 +835,7 @@ bfi_status bfi_integrate(bfi_ctx *ctx, const bfi_lattice *lattice, int64_t nsub,
                  n_slots = at.totals - at.slots, n_totals = sizeof(double) * bfi_totals_len(lattice->nx);
     const size_t up = sub_id ? at.up_end : at.sid, from = replan ? 0 : at.lo;
     const size_t down = slots ? n_slots + n_totals : n_totals;
-    if (up <= kStageBytes && ++ctx->small_jobs == 2) {
+    if ((up <= kStageBytes || down <= kStageBytes) && ++ctx->small_jobs == 2) {
         void *locked = nullptr;
         if (cudaMallocHost(&locked, 2 * kStageBytes) == cudaSuccess) {
             std::free(ctx->stage);
