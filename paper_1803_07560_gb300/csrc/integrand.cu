@@ -46,9 +46,7 @@ namespace bfi {
 // since a CTA's warps share the SM's FP64 pipe.
 constexpr int kMergeSpread = 152;
 constexpr int kMergeThreads = 512, kMergeWarps = kMergeThreads / 32;
-// kexp of a weightless subvolume, and of one whose |ls| is beyond kFarLog or not finite (see finish_subvolume)
-constexpr int kNoWeight = INT_MIN, kFar = INT_MAX;
-constexpr double kFarLog = 0x1p29;
+constexpr int kFarLog = (1023 + 60) << 20;  // upper word of 2^60 (see finish_subvolume)
 
 __device__ __forceinline__ double warp_sum_f64(double v) {
 #pragma unroll
@@ -105,13 +103,14 @@ __device__ __forceinline__ double merge_list(int64_t count, int R, At at, Put pu
 
 // The slot of a subvolume (its sums are in slot[3 ...], unscaled products
 // Q_r = d P_r) and what the totals need of it:
-//   ls = log V - log n - m = kexp ln 2 + ln t, t in [2^-1/2, 2^1/2], so
-//   that f_s / 2^kmax = t 2^(kexp - kmax) once the largest kexp is known;
+//   ls = log V - log n - m = k ln 2 + ln t, so that f_s / 2^kmax =
+//   t 2^(k - kmax) once the largest k is known;
 //   f_buf[s] = t, f_buf[nsub + s] = t^2 / (n - 1), and, in the place of the
-//   subvolume's first chunk record, kexp, V_Z, V_N(r), Cov(r) without f, and ls.
-// An ls that has no such kexp (a box without volume, or an action that leaves
-// |ls| >= kFarLog, as tiny D do) makes merge_slots take f_s = exp(ls - max ls)
-// of every subvolume itself.
+//   subvolume's first chunk record, k, V_Z, V_N(r) and Cov(r) without f.
+// k is an integer in a double: t lies in [2^-1/2, 2^1/2], but for |ls| near 2^60,
+// as tiny D can make it, where k's own rounding leaves it in e^+-200.  From there
+// on two ls are equal or further apart than any weight, so t = 1 and k = 2 ls
+// orders them (above every k below), a box without volume (-inf) included.
 __device__ __forceinline__ void finish_subvolume(const MergeArgs &a, int64_t s, double m) {
     const int lane = threadIdx.x & 31, R = a.R, K = sum_count(R);
     double *slot = a.slots + s * (K + 3);
@@ -149,18 +148,15 @@ __device__ __forceinline__ void finish_subvolume(const MergeArgs &a, int64_t s, 
     }
     __syncwarp();
     const double sw = slot[3], sw2 = slot[4];
-    double tt = 0.0, gt = 0.0, ls = 0.0;
-    int kexp = kNoWeight;
+    double tt = 0.0, gt = 0.0, k = 0.0;
     if (n > 0.0 && sw > 0.0) {
-        ls = log_vol - log_n - m;
-        if (fabs(ls) < kFarLog) {
-            // ln 2 in two parts, the upper one of 32 bits (Cody & Waite's reduction): ls - k upper is exact
-            const double k = rint(ls * 1.4426950408889634);
+        const double ls = log_vol - log_n - m;
+        k = 2.0 * ls;
+        tt = 1.0;
+        if ((__double2hiint(ls) & 0x7fffffff) < kFarLog) {
+            // ln 2 in two parts, the upper one of 32 bits (Cody & Waite's reduction)
+            k = rint(ls * 1.4426950408889634);
             tt = exp(fma(-k, 1.9082149292705877e-10, fma(-k, 0.69314718036912382, ls)));
-            kexp = static_cast<int>(k);
-        } else {
-            kexp = kFar;
-            tt = 1.0;
         }
         if (n >= 2.0) gt = tt * tt / (n - 1.0);
     }
@@ -171,9 +167,8 @@ __device__ __forceinline__ void finish_subvolume(const MergeArgs &a, int64_t s, 
         a.f_buf[s] = tt;
         a.f_buf[a.nsub + s] = gt;
         if (room) {
-            q[0] = static_cast<double>(kexp);
+            q[0] = k;
             q[1] = n * sw2 - sw * sw;
-            q[2 + 2 * R] = ls;
         }
     }
     for (int r = lane; r < R; r += 32) {
@@ -196,30 +191,20 @@ __device__ __forceinline__ void finish_subvolume(const MergeArgs &a, int64_t s, 
 // each, a warp takes 32 / rp subvolumes at a time, rp >= R lanes for each.
 __device__ void merge_slots(const MergeArgs &a) {
     __shared__ double sh[5][kMergeWarps], part[kMergeWarps][32], s_all[5], s_c[32];
-    __shared__ int s_kmax;
+    __shared__ long long s_key;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int R = a.R, K = sum_count(R), SL = K + 3;
     const int64_t nsub = a.nsub;
     auto record = [&](int64_t s) { return a.partials + a.chunk_off[s] * (K + 2); };
-    if (tid == 0) s_kmax = kNoWeight;
+    if (tid == 0) s_key = LLONG_MIN;
     __syncthreads();
-    int kmax = kNoWeight;
+    long long key = LLONG_MIN;
     for (int64_t s = tid; s < nsub; s += kMergeThreads)
-        if (!is_zero(__ldcg(a.f_buf + s))) kmax = max(kmax, static_cast<int>(__ldcg(record(s))));
-    if (kmax != kNoWeight) atomicMax(&s_kmax, kmax);
+        if (!is_zero(__ldcg(a.f_buf + s))) key = max(key, order_f64(__ldcg(record(s))));
+    if (key != LLONG_MIN) atomicMax(&s_key, key);
     __syncthreads();
-    kmax = s_kmax;
-    double lmax = -INFINITY;
-    if (kmax == kFar) {
-        for (int64_t s = tid; s < nsub; s += kMergeThreads)
-            if (!is_zero(__ldcg(a.f_buf + s))) lmax = fmax(lmax, __ldcg(record(s) + 2 + 2 * R));
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) lmax = fmax(lmax, __shfl_xor_sync(0xffffffffu, lmax, off));
-        if (lane == 0) sh[0][warp] = lmax;
-        __syncthreads();
-        for (int w = 0; w < kMergeWarps; ++w) lmax = fmax(lmax, sh[0][w]);
-        __syncthreads();
-    }
+    key = s_key;  // LLONG_MIN: no subvolume has weight
+    const double kmax = unorder_f64(key);
     double z = 0.0, vz = 0.0;
     unsigned long long n_tot = 0;
     int used = 0, bad = 0;
@@ -230,13 +215,12 @@ __device__ void merge_slots(const MergeArgs &a) {
         used += n > 0;
         if (!is_zero(f)) {
             const double *q = record(s);
-            if (kmax == kFar) {
-                f = exp(__ldcg(q + 2 + 2 * R) - lmax);
-                g = n < 2 ? 0.0 : f * f / (static_cast<double>(n) - 1.0);
+            const double k = __ldcg(q) - kmax;
+            if (k >= -1100.0) {
+                f *= pow2(static_cast<int>(k));
+                g *= pow2(2 * static_cast<int>(k));
             } else {
-                const int k = static_cast<int>(__ldcg(q)) - kmax;
-                f *= pow2(k);
-                g *= pow2(2 * max(k, -1100));
+                f = g = k < 0.0 ? 0.0 : NAN;  // no finite kmax, or an ls that is no number
             }
             z = fma(f, __ldcg(a.slots + s * SL + 3), z);
             if (n < 2) bad = 1;
@@ -289,9 +273,8 @@ __device__ void merge_slots(const MergeArgs &a) {
     if (warp == 1 && lane < 2) {  // beside the products' sums of the other warps
         const double Z = s_all[0];
         if (lane == 0)
-            a.totals[0] = kmax == kNoWeight ? -INFINITY
-                          : kmax == kFar    ? lmax + log(Z)
-                                            : fma(static_cast<double>(kmax), 0.69314718055994531, log(Z));
+            a.totals[0] = key == LLONG_MIN ? -INFINITY
+                                              : fma(kmax, fabs(kmax) < 0x1p61 ? 0.69314718055994531 : 0.5, log(Z));
         else
             a.totals[1] = inf_err ? INFINITY : sqrt(s_all[1] > 0.0 ? s_all[1] : 0.0) / Z;
         a.totals[2 + lane] = s_all[2 + lane];

@@ -1,6 +1,6 @@
-"""Totals where the actions are so large that log V - log n - m is far outside
-the range of an exponent times ln 2 (tiny D), and at the range's edge: against
-the estimator's definition on the records."""
+"""Totals where the actions are so large (tiny D) that log V - log n - m is far
+outside the range of an integer exponent, and where its form changes (2^60):
+against the estimator's definition on the records."""
 import numpy as np
 import pytest
 
@@ -12,7 +12,7 @@ torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("D", [2.0 ** -k for k in (8, 18, 22, 23, 24, 25, 26, 30, 45, 100, 400)])
+@pytest.mark.parametrize("D", [2.0 ** -k for k in (8, 18, 22, 23, 24, 25, 26, 30, 45, 48, 49, 50, 51, 52, 53, 54, 55, 100, 400)])
 @pytest.mark.parametrize("precision", [0, 1])
 def test_large_actions(bfi, D, precision):
     """Subvolumes 0 and 3 are the same job; the others' weights are of other orders altogether."""
