@@ -200,7 +200,7 @@ __device__ __forceinline__ float unorder_f32(int b) { return __int_as_float(b ^ 
 // interval of that sample is wider than kMapResolved, the margin that moves a
 // shift, as in slabs close to +-1): every sample of the subvolume is then
 // evaluated.  So it is where the screen gains nothing: where more than 15 in 16
-// of these samples lie within the window of the reference, or more than half
+// of the first 256 lie within the window of the reference, or more than half
 // while the interval is wider than 8, which leaves most threads open.
 // Measured on GB300 at nu = 6 (2^20 to 2^24 samples, intervals of 0.1 to 8):
 // 10x2 20.4 ms at a limit of 0.05 against 0.80 ms at 1, 4 and 16; 32x2 4.95 ms
@@ -216,7 +216,6 @@ __global__ void __launch_bounds__(kBlock) hint_transform(const IntegrandArgs arg
     constexpr int D = NX * NT, NQ = (D + 3) / 4;
     __shared__ int s_min, s_low, s_bad;
     __shared__ unsigned s_unbound, s_near;
-    __shared__ float s_S[4096];  // S_lo of the samples
     __shared__ MapBox s_map[D];
     __shared__ PhiloxPrefix s_pre[NQ + 1];
     const int64_t s = blockIdx.x;
@@ -237,28 +236,32 @@ __global__ void __launch_bounds__(kBlock) hint_transform(const IntegrandArgs arg
     }
     __syncthreads();
     const uint32_t n = static_cast<uint32_t>(hint_samples(args.samples[s]));
-    float mn = INFINITY, ln = INFINITY;
+    float mn = INFINITY, ln = INFINITY, lo_first = INFINITY;
     for (uint32_t k = tid; k < n; k += kBlock) {
         float lo, hi;
         transform_screen<NX, NT>(k, s_pre, rk, s_map, lc, lo, hi);
-        s_S[k] = lo;
+        if (k == static_cast<uint32_t>(tid)) lo_first = lo;
         mn = fminf(mn, hi);
         if (lo == -INFINITY)
             atomicAdd(&s_unbound, 1u);
         else
             ln = fminf(ln, lo);
     }
-    atomicMin(&s_min, order_f32(mn));
-    atomicMin(&s_low, order_f32(ln));
+    // a warp's result first: 256 atomics on one word would take longer than a short hint's samples
+    const int w_min = __reduce_min_sync(0xffffffffu, order_f32(mn)), w_low = __reduce_min_sync(0xffffffffu, order_f32(ln));
+    if ((tid & 31) == 0) {
+        atomicMin(&s_min, w_min);
+        atomicMin(&s_low, w_low);
+    }
     __syncthreads();
     const float best = unorder_f32(s_min), width = best - unorder_f32(s_low);
-    unsigned near = 0u;
-    for (uint32_t k = tid; k < n; k += kBlock) near += s_S[k] > __fadd_ru(best, args.skip_window) ? 0u : 1u;
-    atomicAdd(&s_near, near);
+    const unsigned near = __ballot_sync(0xffffffffu, !(lo_first > __fadd_ru(best, args.skip_window)));
+    if ((tid & 31) == 0) atomicAdd(&s_near, __popc(near));
     __syncthreads();
     if (tid == 0) {
-        const bool bad = s_bad || 256u * s_unbound > n || !(width <= kMapResolved) || 16u * s_near > 15u * n ||
-                         (width > 8.f && 2u * s_near > n);
+        const unsigned of = min(n, static_cast<uint32_t>(kBlock));
+        const bool bad = s_bad || 256u * s_unbound > n || !(width <= kMapResolved) || 16u * s_near > 15u * of ||
+                         (width > 8.f && 2u * s_near > of);
         args.hint[s] = bad ? INFINITY : best;
     }
 }
